@@ -2,6 +2,7 @@
 // launch sequence of each call. All numerical work runs in the kernels of fdlbm_step.cu.
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -10,11 +11,10 @@
 #include <string>
 
 #include "../../include/fdlbm.h"
+#include "fdlbm_fx.cuh"
 #include "fdlbm_internal.h"
 
 using namespace fdlbm;
-
-
 
 namespace {
 
@@ -94,6 +94,21 @@ Layout layout_of(const fdlbm_config* c) {
   return L;
 }
 
+// IEEE binary128 (the same bits on x86-64 and Arm), for what rounding takes from a constant.
+#if LDBL_MANT_DIG == 113
+typedef long double quad;
+#else
+typedef __float128 quad;
+#endif
+
+long long quad_round(quad x) { return (long long)(x < 0 ? x - (quad)0.5 : x + (quad)0.5); }
+// sqrt(1/2): FP64's root refined by Newton's iteration
+quad quad_sqrt_half() {
+  quad y = std::sqrt(0.5);
+  for (int i = 0; i < 2; ++i) y = (y + (quad)0.5 / y) / 2;
+  return y;
+}
+
 // Host-side constants of Eqs. 11 and 17 (FP64).
 Coeffs make_coeffs(const fdlbm_config* cfg) {
   Coeffs c;
@@ -110,6 +125,15 @@ Coeffs make_coeffs(const fdlbm_config* cfg) {
     c.Fh[k][2] = -6.0 * (a + b + cc) / D;
     c.Fh[k][1] = (a * b + b * cc + cc * a) / D;
     c.Fh[k][0] = -(a * b * cc) / (4.0 * D);
+    {  // the same from the speeds' decimals
+      auto sq = [](int i) { return (quad)speed_c(i) * speed_c(i) / 10000; };
+      const quad q = sq(k), qa = sq((k + 1) % 4), qb = sq((k + 2) % 4), qc = sq((k + 3) % 4);
+      const quad qD = q * (q - qa) * (q - qb) * (q - qc);
+      c.Fl[k][3] = (float)(double)(48 / qD - c.Fh[k][3]);
+      c.Fl[k][2] = (float)(double)(-6 * (qa + qb + qc) / qD - c.Fh[k][2]);
+      c.Fl[k][1] = (float)(double)((qa * qb + qb * qc + qc * qa) / qD - c.Fh[k][1]);
+      c.Fl[k][0] = (float)(double)(-(qa * qb * qc) / (4 * qD) - c.Fh[k][0]);
+    }
     c.v[k] = v[k];
     c.v2[k] = vk2;
     c.v3_6[k] = vk2 * v[k] / 6.0;
@@ -159,6 +183,64 @@ Coeffs make_coeffs(const fdlbm_config* cfg) {
     split(c.v4_24[k], c.dv4_24[k]);
     for (int i = 0; i < 4; ++i) split(c.Fh[k][i], c.dFh[k][i]);
   }
+  // Integer weights of the FP64-storage step: units of 2^-S with the sum of a stencil's |weights| (1 - r
+  // among them) below 2^(58 - S), S at most 59. nu is allowed 0.05 lambda, between 1/32 and 1/8.
+  {
+    double most = 0.0;
+    for (int k = 0; k < 4; ++k) {
+      double ax[2][2];
+      for (int a = 0; a < 2; ++a)
+        for (int l = 0; l < 2; ++l)
+          ax[a][l] = std::fabs(c.W1[a][k][l]) + std::fabs(c.Wm1[a][k][l]) + 2.0 * std::fabs(c.D[a][k][l]) +
+                     std::fabs(c.W1[a][k][l] + c.Wm1[a][k][l]);
+      most = std::fmax(most, std::fmax(ax[0][0], ax[1][0]));
+      most = std::fmax(most, ax[0][1] + ax[1][1]);
+    }
+    most += std::fabs(1.0 - cfg->dt / cfg->tau);
+    const double room = std::fmin(std::fmax(0.05 * cfg->lambda, 1.0 / 32), 1.0 / 8);
+    int e = 0;
+    std::frexp(most + 8.0 * room, &e);  // most + 8 room < 2^e
+    const int S = 58 - e < 59 ? 58 - e : 59;
+    if (S >= 55) {
+      c.xS = S;
+      c.xnu = (std::ldexp(1.0, 58 - S) - most) / 8.5;
+      if (c.xnu > 0.5) c.xnu = 0.5;
+      // from the speeds' decimals, like the moments and f_eq's brackets: a flux by other speeds than the
+      // momentum's would differ from it by 2^-53 of f in every step
+      const quad one = 1, half_s = quad_sqrt_half();
+      auto fixed = [&](quad w) { return quad_round(w * (quad)std::ldexp(1.0, S)); };
+      for (int k = 0; k < 4; ++k) {
+        for (int a = 0; a < 2; ++a)
+          for (int l = 0; l < 2; ++l) {
+            const quad cc = (quad)speed_c(k) / 100 * (l == 0 ? one : half_s) * (quad)cfg->dt / (quad)(a == 0 ? cfg->dx : cfg->dy);
+            const quad c2h = lw ? cc * cc / 2 : (quad)0, d = disp ? cc * (1 - cc * cc) / 12 : (quad)0;
+            c.xW1[a][k][l] = fixed(-cc / 2 + c2h - 2 * d);
+            c.xWm1[a][k][l] = fixed(cc / 2 + c2h + 2 * d);
+            const long long di = fixed(d);
+            c.xD[a][k][l][0] = (int)(di >> 28);
+            c.xD[a][k][l][1] = (int)(di & 0xfffffff);
+          }
+        c.xC2[k][0] = c.xW1[0][k][0] + c.xWm1[0][k][0];
+        c.xC2[k][1] = c.xW1[1][k][0] + c.xWm1[1][k][0];
+        c.xC2[k][2] = c.xW1[0][k][1] + c.xWm1[0][k][1] + c.xW1[1][k][1] + c.xWm1[1][k][1];
+      }
+      c.xkeep = std::llrint(std::ldexp(1.0 - cfg->dt / cfg->tau, S));
+    }
+  }
+  // V = 100 v_k is an integer, so the ring constants are exact rationals V^i / den, rounded to 62 bits
+  auto frac = [](int V, int power, unsigned long long den, int e) {
+    unsigned __int128 n = 1;
+    for (int i = 0; i < power; ++i) n *= (unsigned)V;
+    return (long long)(((n << (62 - e)) + den / 2) / den);
+  };
+  for (int own = 0; own < 2; ++own)
+    for (int k = 0; k < 4; ++k) {
+      const int V = speed_c(k), e = own ? k : 3;
+      c.fxc[own][k][0] = frac(V, 2, 20000ull, fx::exp_c1(e));
+      c.fxc[own][k][1] = frac(V, 4, 2400000000ull, fx::exp_c2(e));
+      c.fxc[own][k][2] = frac(V, 1, 100ull, fx::exp_c3(e));
+      c.fxc[own][k][3] = frac(V, 3, 6000000ull, fx::exp_c4(e));
+    }
   split(c.r, c.dr);
   split(s, c.dkS);
   c.sdt = cfg->dt;
@@ -172,15 +254,29 @@ int default_variant(const fdlbm_config* c) {
   const long long sites = (long long)c->nx * c->ny;
   if (c->prec == FDLBM_FNEQ32) return c->ny <= 4 ? V_T32x4 : V_T32x8;  // its own kernel (fdlbm_fneq.cu)
   if (c->prec == FDLBM_FP32_STORE_DW) return V_TMA32x8;  // fastest at every size measured (tiny grids: 32 x 8)
-  // Small grids are latency-bound: four lanes per node win up to a few thousand sites (400 x 4:
-  // 16 us per step against 32 us for the tiles), and lose by 1.3x at 16 000 sites, where the
-  // tiles have reached their latency floor while the ring-parallel launch is throughput-bound.
+  if (c->prec == FDLBM_FP64) {
+    // Small grids are latency-bound: four lanes per node win up to a few thousand sites (400 x 4:
+    // 16 us per step against 32 us for the tiles), and lose by 1.3x at 16 000 sites, where the
+    // tiles have reached their latency floor while the ring-parallel launch is throughput-bound.
+    if (sites <= 6144) return V_RP8x4;
+    // 4-row tubes: a 32 x 16 tile, whose phase 1 takes one round, is fastest up to ~16 000 sites, 16 x 4 up to
+    // ~32 000, then 32 x 4.
+    if (c->ny <= 4) return sites <= 16000 ? V_T32x16 : sites <= 32000 ? V_T16x4 : V_T32x4;
+    return sites < 200000 ? V_T32x8 : V_T32x16;
+  }
+  // FP32 storage, times per step on a GB300 (us). Small grids are latency-bound: four lanes per node win up to
+  // a few thousand sites (400 x 4: 10.3 against 16.4 with tiles; 2000 x 4: 14.4 against 16.4).
   if (sites <= 6144) return V_RP8x4;
-  // 4-row tubes (autotuned on a GB300, FP64 and FP32 storage): a 32 x 16 tile, whose phase 1
-  // takes one round, is fastest up to ~16 000 sites, 16 x 4 up to ~32 000, then 32 x 4.
-  if (c->ny <= 4) return sites <= 16000 ? V_T32x16 : sites <= 32000 ? V_T16x4 : V_T32x4;
-  if (sites < 200000) return V_T32x8;
-  return V_T32x16;
+  // 4-row tubes: the staged 32 x 16 tile, whose phase 1 takes one round, up to 32 000 sites (8000 x 4: 18.4,
+  // 32 x 4 22.5), then 32 x 4 (16384 x 4: 26.6 against 32.8).
+  if (c->ny <= 4) return sites <= 32000 ? V_T32x16 : V_T32x4;
+  // 16 x 4 (128^2: 16.5, 32 x 4 20.5), 32 x 4 (200^2: 24.6, 16 x 4 28.3), the staged 32 x 8 tile (500 x 200: 33.2,
+  // 32 x 4 40.8; 517 x 333: 51.4, tensor copy 52.6), and where tiles come in many waves the tensor copy
+  // (1023 x 777: 173.5 against 179.9; 4096^2: 3280 against 3320, 32 x 16 3470).
+  if (sites <= 20000) return V_T16x4;
+  if (sites <= 60000) return V_T32x4;
+  if (c->ny <= 24) return sites < 200000 ? V_T32x8 : V_T32x16;  // a y-periodic height that one tile may hold
+  return sites <= 300000 ? V_T32x24 : V_TMA32x8;
 }
 
 }  // namespace fdlbm

@@ -54,6 +54,7 @@ struct Grid {
 struct Coeffs {
   // Eq. 11 in Horner form: F_k(th) = th*(h[k][0] + th*(h[k][1] + th*(h[k][2] + th*h[k][3]))).
   double Fh[4][4];
+  float Fl[4][4];     // what rounding took from Fh: the exact coefficient minus Fh (FP64 storage)
   double v[4];        // speeds v_1..v_4
   double v2[4];       // v_k^2
   double v3_6[4];     // v_k^3 / 6
@@ -78,6 +79,16 @@ struct Coeffs {
   float dv[4][2], dv2h[4][2], dv3_6[4][2], dv4_24[4][2];
   // ... and of the F_k polynomials' coefficients, dt/tau and sqrt(1/2)
   float dFh[4][4][2], dr[2], dkS[2];
+  // v_k^2/2, v_k^4/24, v_k, v_k^3/6 as 62-bit fractions of the powers of two of fdlbm_fx.cuh (exp_c1..):
+  // [0] of ring 4's for all rings, [1] of each ring's own
+  long long fxc[2][4][4];
+  // FP64 storage: the weights above (without line IV) as integers in units of 2^-xS (xS = 0: they do not fit
+  // and the FP64 form runs), xC2 the sum of the neighbours' weights; xkeep the weight 1 - r that the
+  // relaxation leaves the node's own value (0 for dt = tau); xnu the largest |nu| the integers allow.
+  long long xW1[2][4][2], xWm1[2][4][2], xC2[4][3], xkeep;
+  int xD[2][4][2][2];  // d as limbs (h, l) of radix 2^28
+  double xnu;
+  int xS;
   // The raw dt, tau, dx, dy: FDLBM_FP64_STRICT forms every ratio itself, in its own order.
   double sdt, stau, sdr[2];
 };
@@ -104,9 +115,8 @@ inline void variant_tile(int v, int* tw, int* th) {
 
 // Launch configuration of the fused step: tile of TW x TH nodes per CTA, registers capped at 128
 // per thread (2-4 CTAs per SM). Phase 1 computes the moments of the tile and its 1-node ring,
-// (TW+2)(TH+2) - 4 nodes, in rounds of one node per thread. 32 x 24 and 32 x 28 on 128 threads
-// fill 98-99 % of their rounds (32 x 16 on 256 threads: 79 %); which shape is fastest depends on
-// the precision and the grid, and the autotuner measures it.
+// (TW+2)(TH+2) - 4 nodes, in rounds of one node per thread. Which shape is fastest depends on the precision
+// and the grid, and the autotuner measures it.
 // V_RP* are the ring-parallel variants (four lanes per node) for small grids; batches use the
 // tile variants only (V_TILE_COUNT).
 // V_S* split the step in two launches: k_moments writes every node's moments once to the grid's

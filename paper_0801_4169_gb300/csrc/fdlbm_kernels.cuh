@@ -8,7 +8,8 @@
 //   moments n, u, T, P of Eqs. 3-5            (tile + 1-node ring, staged in shared memory; FP64
 //                                              sums, or exact fixed-point sums for FP32 storage)
 //   switch theta_alphaI (Eq. 16), kappa (Eq. 15)
-//   weights F_k(theta) (Eqs. 11-13) and f_eq (Eq. 10)        (FP64)
+//   weights F_k(theta) (Eqs. 11-13) and f_eq (Eq. 10)        (FP64; with FP32 storage the brackets of
+//                                              Eq. 10 in 62-bit fixed point, fdlbm_fx.cuh)
 //   Eq. 17 for all 33 velocities, both axes, relaxation once  (storage precision)
 // and writes f_new plus the ghost copies it owns (periodic wrap, zero-gradient copy, specular
 // mirror), so the next step needs no separate boundary pass. With FP32 storage the 32 x 16 and
@@ -22,14 +23,18 @@
 //     FP32 storage the ring, speed-weighted momentum and energy sums are exact 64-bit integers,
 //     and only sqrt(1/2), the two energy parts' sum and 1/100, 10^-4 are applied in FP64;
 //   * f_eq by the even/odd split of each opposite-direction pair: with x = p^2,
-//       nF_k E = alpha + x (beta + gamma x),  nF_k O = p (delta + eps x),  f_eq(+-) = nF_k (E +- O),
-//     where (alpha..eps) are 5 per-ring constants (6 ops per ring, 4 per pair);
+//       nF_k E = alpha + x (beta + gamma x),  nF_k O = p (delta + eps x),  f_eq(+-) = nF_k (E +- O).
+//     FP32 storage forms E and O of a pair in fixed point on the integer pipes, which leaves the site's
+//     constants and the weights, about 60 operations, to the FP64 pipe (4096^2: 4.82 ms per step with
+//     the brackets in FP64, bound by that pipe; 3.47 with the same 32 x 16 tile, 3.28 with the tensor copy,
+//     now bound by the issue of integer multiply-adds);
 //   * dt/tau and n folded into the weights' polynomials, so r*f_eq costs nothing extra;
 //   * the Eq. 17 weights of the +-1 neighbours combined with the node's viscosity once per
 //     (axis, |c| class, ring), shared by the 2-4 directions of that class.
 #include <atomic>
 #include <type_traits>
 
+#include "fdlbm_fx.cuh"
 #include "fdlbm_internal.h"
 
 namespace fdlbm {
@@ -93,6 +98,14 @@ __device__ __forceinline__ float f64_to_f32_rn(double x) {
   return __uint_as_float(t | (hi & 0x80000000u));
 }
 
+// x with its 29 low significand bits dropped, as an FP32 number (exact for |x| in the FP32 normal
+// range); 0 below 2^-126, far under any equilibrium value the scheme adds to others.
+__device__ __forceinline__ float f64_trunc32(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned ah = hi & 0x7fffffffu;
+  const unsigned t = ((ah - (896u << 20)) << 3) | (lo >> 29);
+  return __uint_as_float(ah < (897u << 20) ? 0u : (t | (hi & 0x80000000u)));
+}
 // 1/x for x in the FP32 normal range: an FP32 seed (relative error e ~ 2^-23) refined by one
 // third-order Newton step y (1 + e + e^2), e = 1 - x y, leaving O(e^3) ~ 2^-69: full FP64
 // accuracy up to the last-bit rounding, in 3 FMAs. Outside that range: IEEE division, in a
@@ -347,20 +360,7 @@ __device__ __forceinline__ long long to_fix(float x, int emax) {
   return (long long)t.sm * t.p;
 }
 // V * 2^e2, rounded to nearest even, built from the integer's bits (|V| < 2^63, normal result).
-__device__ __forceinline__ double fix_to_f64(long long V, int e2) {
-  if (V == 0) return 0.0;
-  const unsigned long long sgn = (unsigned long long)V & 0x8000000000000000ull;
-  const unsigned long long A = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
-  const int lz = __clzll((long long)A);  // >= 1
-  const unsigned long long U = A << (lz - 1);  // leading one at bit 62
-  // round to nearest even at bit 10: add 2^9 - 1 plus the lowest kept bit, then drop the 10 bits
-  // (no overflow: U < 2^63). M has its leading one at bit 52, or is 2^53 after a carry.
-  const unsigned long long M = (U + 0x1ffull + ((U >> 10) & 1ull)) >> 10;
-  const unsigned long long E = (unsigned long long)(1086 - lz + e2);  // biased exponent
-  // the leading one (bit 52) adds the last 1 to the exponent field; a carry to 2^53 adds one more,
-  // which is the correct result
-  return __longlong_as_double((long long)(sgn | (((E - 1ull) << 52) + M)));
-}
+__device__ __forceinline__ double fix_to_f64(long long V, int e2) { return fx::to_f64(V, e2); }
 struct RingFix {
   long long S, AX, DX, AY, DY;
 };
@@ -372,11 +372,11 @@ __device__ __forceinline__ RingFix ring_fix(const float (&x)[8], int emax) {
   RingFix r;
   r.S = 0;
 #pragma unroll
-  for (int d = 0; d < 8; ++d) r.S += (long long)t[d].sm * t[d].p;
-  r.AX = (long long)t[7].sm * t[7].p - (long long)t[3].sm * t[3].p;
-  r.AY = (long long)t[1].sm * t[1].p - (long long)t[5].sm * t[5].p;
-  const long long a = (long long)t[0].sm * t[0].p - (long long)t[4].sm * t[4].p;
-  const long long b = (long long)t[6].sm * t[6].p - (long long)t[2].sm * t[2].p;
+  for (int d = 0; d < 8; ++d) r.S = fx::mad(t[d].sm, t[d].p, r.S);
+  r.AX = fx::mad(t[3].sm, -t[3].p, fx::mad(t[7].sm, t[7].p, 0));
+  r.AY = fx::mad(t[5].sm, -t[5].p, fx::mad(t[1].sm, t[1].p, 0));
+  const long long a = fx::mad(t[4].sm, -t[4].p, fx::mad(t[0].sm, t[0].p, 0));
+  const long long b = fx::mad(t[2].sm, -t[2].p, fx::mad(t[6].sm, t[6].p, 0));
   r.DX = a + b;
   r.DY = a - b;
   return r;
@@ -390,9 +390,9 @@ __device__ __forceinline__ Mom nan_moments() {
 // as hi 2^32 + lo (lo unsigned): EH = sum_k V_k^2 hi_k (|EH| < 2^41) and EL = sum_k V_k^2 lo_k
 // (< 2^52) are exact integers.
 __device__ __forceinline__ void energy_parts(int k, long long S, long long& EH, long long& EL) {
-  const long long v2 = (long long)speed_c(k) * speed_c(k);
-  EH += v2 * (long long)(int)(S >> 32);
-  EL += v2 * (long long)(unsigned)S;
+  const int v2 = speed_c(k) * speed_c(k);
+  EH = fx::mad((int)(S >> 32), v2, EH);
+  EL = fx::mad_u((unsigned)S, (unsigned)v2, EL);
 }
 // n, 100 jx, 100 jy and 10^4 sum |v|^2 f from the exact sums. EH 2^32 and EL convert to FP64
 // exactly (both below 2^53), so their one FP64 sum is the correctly rounded energy sum.
@@ -417,10 +417,10 @@ __device__ __forceinline__ Mom fix_node_moments(const float (&x)[Q], int emax) {
     for (int d = 0; d < 8; ++d) g[d] = x[1 + 8 * k + d];
     const RingFix r = ring_fix<FULL>(g, emax);
     N += r.S;
-    Ax += speed_c(k) * r.AX;
-    Dx += speed_c(k) * r.DX;
-    Ay += speed_c(k) * r.AY;
-    Dy += speed_c(k) * r.DY;
+    Ax = fx::mad_small(speed_c(k), r.AX, Ax);
+    Dx = fx::mad_small(speed_c(k), r.DX, Dx);
+    Ay = fx::mad_small(speed_c(k), r.AY, Ay);
+    Dy = fx::mad_small(speed_c(k), r.DY, Dy);
     energy_parts(k, r.S, EH, EL);
   }
   return fix_moments(N, Ax, Dx, Ay, Dy, EH, EL, e2);
@@ -629,19 +629,127 @@ __device__ __forceinline__ void eq_pair(const EqRing& r, double p, double x, dou
   fp = NE + NO;
   fm = NE - NO;
 }
-template <typename S>
-__device__ __forceinline__ void eq_pair_s(const EqRing& r, double p, double x, S& fp, S& fm);
-template <>
-__device__ __forceinline__ void eq_pair_s<double>(const EqRing& r, double p, double x, double& fp, double& fm) {
-  eq_pair(r, p, x, fp, fm);
+
+// FP32 storage: the even and odd parts of the moving directions' r f_eq in 62-bit fixed point
+// (fdlbm_fx.cuh), each rounded to FP32 once; the pair is formed in FP32, the precision it is stored in.
+struct F8 {
+  float v[8];
+};
+// FP64 form of one ring for nodes outside the fixed-point range (NaN and infinities among them).
+__device__ __noinline__ F8 feq_ring_rare(double n, double ux, double uy, double T, int K, const Coeffs& c) {
+  const EqSite e = eq_site(n, ux, uy, T, c);
+  const EqRing r = eq_ring(e, K, c);
+  F8 o;
+  auto pair = [&](int t, float& plus, float& minus) {
+    double NE, NO;
+    eq_parts(r, e.p[t], e.x[t], NE, NO);
+    const float a = f64_to_f32_rn(NE), b = f64_to_f32_rn(NO);
+    plus = a + b;
+    minus = a - b;
+  };
+  pair(0, o.v[7], o.v[3]);
+  pair(1, o.v[0], o.v[4]);
+  pair(2, o.v[1], o.v[5]);
+  pair(3, o.v[2], o.v[6]);
+  return o;
 }
-template <>
-__device__ __forceinline__ void eq_pair_s<float>(const EqRing& r, double p, double x, float& fp, float& fm) {
-  double NE, NO;
-  eq_parts(r, p, x, NE, NO);
-  const float e = f64_to_f32_rn(NE), o = f64_to_f32_rn(NO);
-  fp = e + o;
-  fm = e - o;
+struct FeqNode {
+  fx::Dir q[4];
+  fx::Base b;
+  fx::Limb A0;   // FP32 storage: A0 2^-es, and es for all rings
+  int es;
+  unsigned neg;  // bit t: projection t is negative
+  double A0d, th, rnth;  // A0, theta, r n theta
+};
+// The site numbers of Eq. 10 that the brackets need: the projections (x, diagonal, y, anti-diagonal), A0, A1
+// and their scales.
+struct FeqSite64 {
+  double p[4], A0;
+  fx::Base b;
+  unsigned neg;
+};
+__device__ __forceinline__ FeqSite64 feq_site64(double ux, double uy, double T) {
+  FeqSite64 o;
+  const double ith = rcp64(T);
+  const double px = ux * ith, py = uy * ith;
+  o.p[0] = px;
+  o.p[1] = kS * (px + py);
+  o.p[2] = py;
+  o.p[3] = kS * (py - px);
+  const double b2 = fma(ux, px, uy * py);  // 2b = |u|^2/theta
+  const double A1 = fma(-0.5, b2, 1.0);
+  o.A0 = fma(0.125 * b2, b2, A1);  // A1 + (2b)^2/8
+  o.b = fx::base_of(o.A0, A1, o.p[0], o.p[1], o.p[2], o.p[3]);
+  o.neg = 0u;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) o.neg |= (unsigned)__double2hiint(o.p[t]) >> 31 << t;
+  return o;
+}
+template <typename S>
+__device__ __forceinline__ FeqNode feq_node(double n, double ux, double uy, double T, const Coeffs& c) {
+  const FeqSite64 s = feq_site64(ux, uy, T);
+  FeqNode o;
+  o.b = s.b;
+  o.neg = s.neg;
+  o.A0d = s.A0;
+  o.th = T;
+  o.rnth = c.r * n * T;
+  if constexpr (std::is_same<S, float>::value) {
+    o.es = fx::scale_of(o.b, 3);
+    o.A0 = fx::limb(o.b.A0f >> fx::imin(o.es - o.b.e0, 63));
+  }
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const fx::Powers w = fx::powers_of(o.b, s.p[t], std::is_same<S, float>::value ? 0 : 2);
+    if constexpr (std::is_same<S, float>::value) o.q[t] = fx::dir_shared(w, o.b, o.es);
+    else o.q[t] = fx::dir_plain(w);
+  }
+  return o;
+}
+// r n F_k (Eqs. 11-13) from r n theta. Where f_eq's brackets and the moments take the speeds as exact
+// decimals (FP64 storage), F_k's coefficients have to be theirs too: rounded to FP64 they violate the moment
+// identities by 2^-53 of f, always with the same sign. The rounded parts' polynomial, in FP32, enters with
+// the last operation.
+template <bool EXACT>
+__device__ __forceinline__ double weight_poly(double rnth, double th, int K, const Coeffs& c) {
+  const double P = fma(th, fma(th, fma(th, c.Fh[K][3], c.Fh[K][2]), c.Fh[K][1]), c.Fh[K][0]);
+  if constexpr (!EXACT) return rnth * P;
+  const float t = f64_trunc32(th), l = fmaf(t, fmaf(t, fmaf(t, c.Fl[K][3], c.Fl[K][2]), c.Fl[K][1]), c.Fl[K][0]);
+  const float corr = f64_trunc32(rnth) * l;
+  const double d = fabsf(corr) >= 1.17549435e-38f ? f32_to_f64_bits(corr) : 0.0;
+  return fma(rnth, P, d);
+}
+template <bool EXACT>
+__device__ __forceinline__ double ring_weight(const FeqNode& e, int K, const Coeffs& c) {
+  return weight_poly<EXACT>(e.rnth, e.th, K, c);
+}
+// direction index (0..7) of projection t (x, diagonal, y, anti-diagonal) and of its opposite
+__device__ constexpr int dir_plus(int t) { return t == 0 ? 7 : t - 1; }
+__device__ constexpr int dir_minus(int t) { return t == 0 ? 3 : t + 3; }
+// r f_eq of ring K's 8 directions; nF = ring_weight<false>(e, K, c). n..T: the node's macros (rare form).
+__device__ __forceinline__ void feq_ring(const FeqNode& e, int K, double nF, const Coeffs& c, double n, double ux,
+                                         double uy, double T, float (&fe)[8]) {
+  if (__builtin_expect(e.b.ok && fx::weight_ok(nF), 1)) {
+    const fx::RingFx r = fx::ring_shared(e.A0, e.es, nF, c.fxc[0][K]);
+    const float up = fx::pow2_f32(r.ex + 36), down = fx::pow2_f32(r.ex + 4);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      long long NE, NO;
+      fx::pair_of<false>(r, e.q[t], NE, NO);
+      const float ev = fx::narrow_f32(NE, up, down);
+      const float od = __uint_as_float(__float_as_uint(fx::narrow_f32(NO, up, down)) ^ ((e.neg >> t) << 31));
+      fe[dir_plus(t)] = ev + od;
+      fe[dir_minus(t)] = ev - od;
+    }
+  } else {
+    const F8 o = feq_ring_rare(n, ux, uy, T, K, c);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) fe[i] = o.v[i];
+  }
+}
+// r f_eq of the rest velocity: r n F_0 A0 with r n F_0 = r n - 8 sum_k r n F_k
+__device__ __forceinline__ float feq_rest(const FeqNode& e, double n, double snF, const Coeffs& c) {
+  return f64_to_f32_rn(fma(-8.0, snF, c.r * n) * e.A0d);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -658,14 +766,6 @@ __device__ __forceinline__ void eq_pair_s<float>(const EqRing& r, double p, doub
 struct dw {
   float h, l;
 };
-// x with its 29 low significand bits dropped, as an FP32 number (exact for |x| in the FP32 normal
-// range); 0 below 2^-126, far under any equilibrium value the scheme adds to others.
-__device__ __forceinline__ float f64_trunc32(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const unsigned ah = hi & 0x7fffffffu;
-  const unsigned t = ((ah - (896u << 20)) << 3) | (lo >> 29);
-  return __uint_as_float(ah < (897u << 20) ? 0u : (t | (hi & 0x80000000u)));
-}
 // x = hi + lo: hi its leading 24 bits, lo the (exact, FP64) remainder truncated to FP32, so
 // |x - hi - lo| < 2^-47 |x|. One FP64 operation.
 __device__ __forceinline__ dw split_dw(double x) {
@@ -915,22 +1015,23 @@ __device__ __forceinline__ void update_ring(int K, const S* __restrict__ f, S* _
       }
     }
   } else {
+    static_assert(std::is_same<S, double>::value, "FP32 storage takes its f_eq from feq_ring");
     const EqRing er = eq_ring(e, K, c);
     S fp, fm;
     // pair (d7: 0 deg, d3: 180 deg), projection p_x
-    eq_pair_s<S>(er, e.p[0], e.x[0], fp, fm);
+    eq_pair(er, e.p[0], e.x[0], fp, fm);
     out[7] = stencil_dir<S, 7, COH>(fq + (long long)(1 + 8 * K + 7) * g.plane, g.pitch, w, fp);
     out[3] = stencil_dir<S, 3, COH>(fq + (long long)(1 + 8 * K + 3) * g.plane, g.pitch, w, fm);
     // pair (d0: 45 deg, d4: 225 deg), projection s(p_x + p_y)
-    eq_pair_s<S>(er, e.p[1], e.x[1], fp, fm);
+    eq_pair(er, e.p[1], e.x[1], fp, fm);
     out[0] = stencil_dir<S, 0, COH>(fq + (long long)(1 + 8 * K + 0) * g.plane, g.pitch, w, fp);
     out[4] = stencil_dir<S, 4, COH>(fq + (long long)(1 + 8 * K + 4) * g.plane, g.pitch, w, fm);
     // pair (d1: 90 deg, d5: 270 deg), projection p_y
-    eq_pair_s<S>(er, e.p[2], e.x[2], fp, fm);
+    eq_pair(er, e.p[2], e.x[2], fp, fm);
     out[1] = stencil_dir<S, 1, COH>(fq + (long long)(1 + 8 * K + 1) * g.plane, g.pitch, w, fp);
     out[5] = stencil_dir<S, 5, COH>(fq + (long long)(1 + 8 * K + 5) * g.plane, g.pitch, w, fm);
     // pair (d2: 135 deg, d6: 315 deg), projection s(p_y - p_x)
-    eq_pair_s<S>(er, e.p[3], e.x[3], fp, fm);
+    eq_pair(er, e.p[3], e.x[3], fp, fm);
     out[2] = stencil_dir<S, 2, COH>(fq + (long long)(1 + 8 * K + 2) * g.plane, g.pitch, w, fp);
     out[6] = stencil_dir<S, 6, COH>(fq + (long long)(1 + 8 * K + 6) * g.plane, g.pitch, w, fm);
   }
@@ -1050,25 +1151,19 @@ __device__ __forceinline__ void stage_feq(S* __restrict__ s_fe, int node, double
     }
     return;
   }
-  const EqSite e = eq_site(n, ux, uy, T, c);
-  s_fe[node] = to_s<S>(e.rest);
-#pragma unroll
+  static_assert(std::is_same<S, float>::value, "only FP32 storage stages f_eq");
+  const FeqNode e = feq_node<S>(n, ux, uy, T, c);
+  double snF = 0.0;
+#pragma unroll 1  // unrolled, the rings' code no longer fits the instruction cache beside the stencils'
   for (int K = 0; K < 4; ++K) {
-    const EqRing er = eq_ring(e, K, c);
-    S fp, fm;
-    eq_pair_s<S>(er, e.p[0], e.x[0], fp, fm);
-    s_fe[(1 + 8 * K + 7) * NN + node] = fp;
-    s_fe[(1 + 8 * K + 3) * NN + node] = fm;
-    eq_pair_s<S>(er, e.p[1], e.x[1], fp, fm);
-    s_fe[(1 + 8 * K + 0) * NN + node] = fp;
-    s_fe[(1 + 8 * K + 4) * NN + node] = fm;
-    eq_pair_s<S>(er, e.p[2], e.x[2], fp, fm);
-    s_fe[(1 + 8 * K + 1) * NN + node] = fp;
-    s_fe[(1 + 8 * K + 5) * NN + node] = fm;
-    eq_pair_s<S>(er, e.p[3], e.x[3], fp, fm);
-    s_fe[(1 + 8 * K + 2) * NN + node] = fp;
-    s_fe[(1 + 8 * K + 6) * NN + node] = fm;
+    const double nF = ring_weight<false>(e, K, c);
+    snF += nF;
+    float fe[8];
+    feq_ring(e, K, nF, c, n, ux, uy, T, fe);
+#pragma unroll
+    for (int d = 0; d < 8; ++d) s_fe[(1 + 8 * K + d) * NN + node] = fe[d];
   }
+  s_fe[node] = feq_rest(e, n, snF, c);
 }
 
 // One node of phase 1: the moments of local node (lx, ly) of the tile whose first node is (x0, y0)
@@ -1151,7 +1246,8 @@ __device__ __forceinline__ void staged_update(const S* __restrict__ f, S* __rest
       acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
       store_node<S, 0>(fn, g, gx, gy, go, acc);
     }
-#pragma unroll
+    constexpr int RINGS = DW ? 4 : 1;
+#pragma unroll RINGS
     for (int K = 0; K < 4; ++K) {
       S fe[8];
 #pragma unroll
@@ -1202,7 +1298,8 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
   } else {
   const bool wrap = WRAPY && y0 == 0 && g.ny <= TH && g.bc[2] == BC_PERIODIC && g.bc[3] == BC_PERIODIC;
   const int nslot = wrap ? SW * g.ny : SW * SH;  // with wrap: local rows 1..ny only
-#pragma unroll
+  constexpr int SLOTS = DW || std::is_same<S, double>::value ? NSLOT : 1;
+#pragma unroll SLOTS
   for (int k = 0; k < NSLOT; ++k) {
     const int idx = tid + k * NT;
     // the slots before the last always lie in the tile ring (no branch); the last one is guarded
@@ -1253,14 +1350,17 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
       snuy = (S)0.5 * thy * aky * ((S)1 - aky);
     }
     const S w0base = ((S)1 - SC::r(c)) - (S)2 * (snux + snuy);
-    using ES = typename std::conditional<DW, EqSiteDW, EqSite>::type;
+    constexpr bool FXQ = std::is_same<S, float>::value && !DW;
+    using ES = typename std::conditional<DW, EqSiteDW, typename std::conditional<FXQ, FeqNode, EqSite>::type>::type;
     ES e;
+    double snF = 0.0;
     if constexpr (DW) e = eq_site_dw(n, ux, uy, T, c);
+    else if constexpr (FXQ) e = feq_node<S>(n, ux, uy, T, c);
     else e = eq_site(n, ux, uy, T, c);
     const long long off = (long long)(gy + NG) * g.pitch + (gx + NG);
     const GhostOwn go = ghost_own(g, gx, gy);
     // rest velocity: f_eq = n F_0 A0; c = 0 on both axes (line IV only)
-    {
+    if constexpr (!FXQ) {
       S rfeq;
       if constexpr (DW) rfeq = e.rest;
       else rfeq = to_s<S>(e.rest);
@@ -1270,10 +1370,26 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
       acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
       store_node<S, 0>(fn, g, gx, gy, go, acc);
     }
-    update_ring<S, ES, COH>(0, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-    update_ring<S, ES, COH>(1, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-    update_ring<S, ES, COH>(2, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-    update_ring<S, ES, COH>(3, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+    if constexpr (std::is_same<S, float>::value && !DW) {
+#pragma unroll 1
+      for (int K = 0; K < 4; ++K) {
+        const double nF = ring_weight<false>(e, K, c);
+        snF += nF;
+        S fe[8];
+        feq_ring(e, K, nF, c, n, ux, uy, T, fe);
+        ring_stencil<S, COH>(K, f, fn, g, c, off, gx, gy, go, fe, w0base, snux, snuy);
+      }
+      const S* p = f + off;
+      S acc = fma(w0base, ldc<COH>(p), feq_rest(e, n, snF, c));
+      acc = fma(snux, ldc<COH>(p + 1) + ldc<COH>(p - 1), acc);
+      acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
+      store_node<S, 0>(fn, g, gx, gy, go, acc);
+    } else {
+      update_ring<S, ES, COH>(0, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, ES, COH>(1, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, ES, COH>(2, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, ES, COH>(3, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+    }
   }
   }
   if (bits) atomicOr(health, bits);
@@ -1307,9 +1423,7 @@ __global__ void __launch_bounds__(BX * BY, MINB) k_update(const S* __restrict__ 
 // Batched step: every member solve of a batch advances one time step in one launch. Members share
 // the scheme constants (dx, dy, dt, tau, lambda, flags, precision), not their grids, boundaries or
 // buffers. Block b runs tile (b - tile0) of the member whose [tile0, tile0 + tiles) holds b.
-template <typename S, int BX, int BY, int RY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB) k_step_batch(const BatchMember* __restrict__ mem, int nmem,
-                                                        unsigned long long step, Coeffs c) {
+__device__ __forceinline__ int batch_member(const BatchMember* __restrict__ mem, int nmem) {
   __shared__ int s_sel;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     const long long b = blockIdx.x;
@@ -1322,7 +1436,12 @@ __global__ void __launch_bounds__(BX * BY, MINB) k_step_batch(const BatchMember*
     s_sel = lo;
   }
   __syncthreads();
-  const BatchMember& m = mem[s_sel];
+  return s_sel;
+}
+template <typename S, int BX, int BY, int RY, int MINB>
+__global__ void __launch_bounds__(BX * BY, MINB) k_step_batch(const BatchMember* __restrict__ mem, int nmem,
+                                                        unsigned long long step, Coeffs c) {
+  const BatchMember& m = mem[batch_member(mem, nmem)];
   const Grid g = m.g;
   const long long local = (long long)blockIdx.x - m.tile0;
   const int tx = (int)(local % m.tiles_x), ty = (int)(local / m.tiles_x);
@@ -1403,18 +1522,33 @@ __device__ __forceinline__ void rp_tile(const S* __restrict__ f, S* __restrict__
       snuy = (S)0.5 * thy * aky * ((S)1 - aky);
     }
     const S w0base = ((S)1 - SC::r(c)) - (S)2 * (snux + snuy);
-    const EqSite e = eq_site(n, ux, uy, T, c);
     const long long off = (long long)(gy + NG) * g.pitch + (gx + NG);
     const GhostOwn go = ghost_own(g, gx, gy);
-    if (r == 0) {
-      const S rfeq = to_s<S>(e.rest);
+    auto rest = [&](S rfeq) {
       const S* p = f + off;
       S acc = fma(w0base, ldc<COH>(p), rfeq);
       acc = fma(snux, ldc<COH>(p + 1) + ldc<COH>(p - 1), acc);
       acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
       store_node<S, 0>(fn, g, gx, gy, go, acc);
+    };
+    if constexpr (std::is_same<S, float>::value) {
+      const FeqNode e = feq_node<S>(n, ux, uy, T, c);
+      double nF = 0.0, snF = 0.0;
+#pragma unroll
+      for (int K = 0; K < 4; ++K) {
+        const double w = ring_weight<false>(e, K, c);
+        snF += w;
+        if (K == r) nF = w;
+      }
+      if (r == 0) rest(feq_rest(e, n, snF, c));
+      S fe[8];
+      feq_ring(e, r, nF, c, n, ux, uy, T, fe);
+      ring_stencil<S, COH>(r, f, fn, g, c, off, gx, gy, go, fe, w0base, snux, snuy);
+    } else {
+      const EqSite e = eq_site(n, ux, uy, T, c);
+      if (r == 0) rest(e.rest);
+      update_ring<S, EqSite, COH>(r, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
     }
-    update_ring<S, EqSite, COH>(r, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
   }
   if (bits) atomicOr(health, bits);
 }

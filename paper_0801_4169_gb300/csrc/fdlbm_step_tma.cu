@@ -8,10 +8,10 @@
 // fixed-point sums), the switch (Eq. 16) and the Eq. 17 stencils then read shared memory at
 // offsets known at compile time, instead of global loads with 64-bit address arithmetic. The
 // arithmetic of every node is that of the other FP32-storage variants, so results are bitwise
-// the same. The equilibrium is formed ring by ring between the stencils (FP64, or double-word
-// FP32 for FDLBM_FP32_STORE_DW). 69 KB of shared memory per CTA: three CTAs per SM. With the
-// double-word equilibrium this is the fastest FP32-storage step (2.42 against 3.11 ms per 4096^2
-// step for the staged 32 x 8 tile); with the FP64 one the FP64 pipe binds and it gains nothing.
+// the same. The equilibrium is formed ring by ring between the stencils (in fixed point, or double-word
+// FP32 for FDLBM_FP32_STORE_DW). 69 KB of shared memory per CTA: three CTAs per SM. The fastest
+// FP32-storage step on large grids: 4096^2 in 3.28 ms against 3.32 for the staged 32 x 8 tile, with the
+// double-word equilibrium 2.42 against 3.11.
 //
 // The box is addressed in padded-grid coordinates: for the tile at node (x0, y0) it starts at
 // padded column x0 (node x0 - 2) and padded row y0, so its first coordinate is a multiple of 32
@@ -117,12 +117,13 @@ __device__ __forceinline__ float box_stencil(const float* __restrict__ p, const 
   return acc;
 }
 
-// The 8 velocities of ring K at one node: their r f_eq (FP64 pairs rounded to FP32, or the
-// double-word pairs), the stencils from the box, and the store with the node's ghost copies.
+// The 8 velocities of ring K at one node: their r f_eq (fixed-point or double-word pairs), the stencils from
+// the box, and the store with the node's ghost copies. snF: the sum of the rings' weights so far.
 template <typename ES>
 __device__ __forceinline__ void box_ring(int K, const float* __restrict__ sp, float* __restrict__ fn, const Grid& g,
                                          const Coeffs& c, int gx, int gy, const GhostOwn& go, const ES& e,
-                                         float w0base, float nux, float nuy) {
+                                         float w0base, float nux, float nuy, double n, double ux, double uy, double T,
+                                         double& snF) {
   using SC = StencilConsts<float>;
   RingW<float> w;
 #pragma unroll
@@ -147,11 +148,9 @@ __device__ __forceinline__ void box_ring(int K, const float* __restrict__ sp, fl
     eq_pair_dw(er, e.p[2], e.x[2], fe[1], fe[5]);
     eq_pair_dw(er, e.p[3], e.x[3], fe[2], fe[6]);
   } else {
-    const EqRing er = eq_ring(e, K, c);
-    eq_pair_s<float>(er, e.p[0], e.x[0], fe[7], fe[3]);
-    eq_pair_s<float>(er, e.p[1], e.x[1], fe[0], fe[4]);
-    eq_pair_s<float>(er, e.p[2], e.x[2], fe[1], fe[5]);
-    eq_pair_s<float>(er, e.p[3], e.x[3], fe[2], fe[6]);
+    const double nF = ring_weight<false>(e, K, c);
+    snF += nF;
+    feq_ring(e, K, nF, c, n, ux, uy, T, fe);
   }
   const float* pk = sp + (1 + 8 * K) * kBP;
   float out[8];
@@ -166,8 +165,7 @@ __device__ __forceinline__ void box_ring(int K, const float* __restrict__ sp, fl
   store_ring<float>(fn, g, gx, gy, go, K, out);
 }
 
-// ROLL: the four rings run as a loop instead of unrolled (a quarter of phase 2's code).
-template <bool DW, int MINB, bool ROLL>
+template <bool DW, int MINB>
 __global__ void __launch_bounds__(kTW * kTH, MINB)
     k_step_tma(const __grid_constant__ CUtensorMap tmap, float* __restrict__ fn, Grid g, Coeffs c,
                unsigned* __restrict__ health) {
@@ -247,30 +245,24 @@ __global__ void __launch_bounds__(kTW * kTH, MINB)
       snuy = 0.5f * thy * aky * (1.f - aky);
     }
     const float w0base = (1.f - SC::r(c)) - 2.f * (snux + snuy);
-    using ES = typename std::conditional<DW, EqSiteDW, EqSite>::type;
+    using ES = typename std::conditional<DW, EqSiteDW, FeqNode>::type;
     ES e;
+    double snF = 0.0;
     if constexpr (DW) e = eq_site_dw(n, ux, uy, T, c);
-    else e = eq_site(n, ux, uy, T, c);
+    else e = feq_node<float>(n, ux, uy, T, c);
     const GhostOwn go = ghost_own(g, gx, gy);
     const float* sp = s_f + (threadIdx.y + NG) * kBW + (threadIdx.x + NG);
-    {
-      float rfeq;
-      if constexpr (DW) rfeq = e.rest;
-      else rfeq = to_s<float>(e.rest);
+    auto rest = [&](float rfeq) {
       float acc = fmaf(w0base, sp[0], rfeq);
       acc = fmaf(snux, sp[1] + sp[-1], acc);
       acc = fmaf(snuy, sp[kBW] + sp[-kBW], acc);
       store_node<float, 0>(fn, g, gx, gy, go, acc);
-    }
-    if constexpr (ROLL) {
+    };
+    if constexpr (DW) rest(e.rest);
+    // a loop: unrolled, the rings' code passes the instruction cache (3.48 ms per 4096^2 step against 3.28)
 #pragma unroll 1
-      for (int K = 0; K < 4; ++K) box_ring<ES>(K, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy);
-    } else {
-      box_ring<ES>(0, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy);
-      box_ring<ES>(1, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy);
-      box_ring<ES>(2, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy);
-      box_ring<ES>(3, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy);
-    }
+    for (int K = 0; K < 4; ++K) box_ring<ES>(K, sp, fn, g, c, gx, gy, go, e, w0base, snux, snuy, n, ux, uy, T, snF);
+    if constexpr (!DW) rest(feq_rest(e, n, snF, c));
   }
   if (bits) atomicOr(health, bits);
 }
@@ -307,17 +299,17 @@ static cudaError_t tile_map(CUtensorMap* map, const void* f, const Grid& g) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <bool DW, bool ROLL>
+template <bool DW>
 static cudaError_t launch_tma_t(const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
                                 cudaStream_t s) {
   CUtensorMap map;
   cudaError_t e = tile_map(&map, f, g);
   if (e != cudaSuccess) return e;
   static std::atomic<unsigned long long> attr{0};  // devices already opted in
-  e = allow_dynamic_smem(k_step_tma<DW, 3, ROLL>, kSmemBytes, attr);
+  e = allow_dynamic_smem(k_step_tma<DW, 3>, kSmemBytes, attr);
   if (e != cudaSuccess) return e;
   dim3 block(kTW, kTH), grid((g.nx + kTW - 1) / kTW, (g.ny + kTH - 1) / kTH);
-  k_step_tma<DW, 3, ROLL><<<grid, block, kSmemBytes, s>>>(map, static_cast<float*>(fn), g, c, health);
+  k_step_tma<DW, 3><<<grid, block, kSmemBytes, s>>>(map, static_cast<float*>(fn), g, c, health);
   return cudaGetLastError();
 }
 
@@ -328,7 +320,7 @@ cudaError_t launch_step_tma(bool dw, const void* f, void* fn, const Grid& g, con
                             cudaStream_t s) {
   if (g.pitch < kBW || g.rows < kBH)
     return dw ? launch_step_f32dw(V_T32x8, f, fn, g, c, health, s) : launch_step_f32(V_T32x8, f, fn, g, c, health, s);
-  return dw ? launch_tma_t<true, true>(f, fn, g, c, health, s) : launch_tma_t<false, false>(f, fn, g, c, health, s);
+  return dw ? launch_tma_t<true>(f, fn, g, c, health, s) : launch_tma_t<false>(f, fn, g, c, health, s);
 }
 
 namespace {
