@@ -58,20 +58,18 @@ cudaError_t launch_step(int prec, int variant, const void* f, void* fn, const Gr
   if (variant == V_TMA32x8) {
     if (prec == FDLBM_FP32_STORE || prec == FDLBM_FP32_STORE_DW)
       return launch_step_tma(prec == FDLBM_FP32_STORE_DW, f, fn, g, c, health, s);
-    variant = V_T32x8;  // FP64 storage: the box would take 114 KB
+    variant = V_T32x8;
   }
   if (prec == FDLBM_FP32_STORE_DW) return launch_step_f32dw(variant, f, fn, g, c, health, s);
+  if (prec == FDLBM_FP64) return launch_step_f64(variant, f, fn, g, c, health, s);
   // a tile that holds a y-periodic grid's whole height reuses the interior rows' moments for its
   // ghost rows (same values, bit for bit)
   if (variant >= 0 && variant < V_TILE_COUNT && g.bc[2] == BC_PERIODIC && g.bc[3] == BC_PERIODIC) {
     int tw, th;
     variant_tile(variant, &tw, &th);
-    if (g.ny <= th)
-      return prec == 0 ? launch_step_wrap_f64(variant, f, fn, g, c, health, s)
-                       : launch_step_wrap_f32(variant, f, fn, g, c, health, s);
+    if (g.ny <= th) return launch_step_wrap_f32(variant, f, fn, g, c, health, s);
   }
-  return prec == 0 ? launch_step_f64(variant, f, fn, g, c, health, s)
-                   : launch_step_f32(variant, f, fn, g, c, health, s);
+  return launch_step_f32(variant, f, fn, g, c, health, s);
 }
 
 cudaError_t launch_gather_health(const BatchMember* mem, int nmem, unsigned* out, cudaStream_t s) {

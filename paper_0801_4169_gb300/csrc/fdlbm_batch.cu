@@ -85,13 +85,14 @@ int rebuild(fdlbm_batch_ctx* b) {
     b->variant = ny <= 4 ? V_T32x4 : ny <= 8 || b->scheme.prec == FDLBM_FNEQ32 ? V_T32x8 : V_T32x16;
   }
   if (n && !variant_ok(b, b->variant)) b->variant = V_T32x8;  // an FNEQ32 batch given another shape
-  if (n && b->scheme.prec == FDLBM_FNEQ32) {
-    const cudaError_t pe = prepare_batch_fneq(b->variant);
+  if (n && (b->scheme.prec == FDLBM_FNEQ32 || b->scheme.prec == FDLBM_FP64)) {
+    const cudaError_t pe =
+        b->scheme.prec == FDLBM_FP64 ? prepare_batch_f64(b->variant) : prepare_batch_fneq(b->variant);
     if (pe != cudaSuccess) return bcuda(b, pe, "batch kernel set-up");
   }
   b->host_table.resize(n);
   int tw, th;
-  variant_tile(b->variant, &tw, &th);
+  batch_tile(b->scheme.prec, b->variant, &tw, &th);
   long long tile0 = 0;
   for (size_t i = 0; i < n; ++i) {
     fdlbm_ctx* h = b->members[i];

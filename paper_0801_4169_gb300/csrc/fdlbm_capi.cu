@@ -255,14 +255,13 @@ int default_variant(const fdlbm_config* c) {
   if (c->prec == FDLBM_FNEQ32) return c->ny <= 4 ? V_T32x4 : V_T32x8;  // its own kernel (fdlbm_fneq.cu)
   if (c->prec == FDLBM_FP32_STORE_DW) return V_TMA32x8;  // fastest at every size measured (tiny grids: 32 x 8)
   if (c->prec == FDLBM_FP64) {
-    // Small grids are latency-bound: four lanes per node win up to a few thousand sites (400 x 4:
-    // 16 us per step against 32 us for the tiles), and lose by 1.3x at 16 000 sites, where the
-    // tiles have reached their latency floor while the ring-parallel launch is throughput-bound.
-    if (sites <= 6144) return V_RP8x4;
-    // 4-row tubes: a 32 x 16 tile, whose phase 1 takes one round, is fastest up to ~16 000 sites, 16 x 4 up to
-    // ~32 000, then 32 x 4.
-    if (c->ny <= 4) return sites <= 16000 ? V_T32x16 : sites <= 32000 ? V_T16x4 : V_T32x4;
-    return sites < 200000 ? V_T32x8 : V_T32x16;
+    // Times per step on a GB300 (us). The 4 x 4 tile (V_RP8x4; two per SM, 4864 sites at a time) is the shortest
+    // step: 400 x 4 9.7 against 13.9 with 8 x 4 tiles, 2000 x 4 18.4 against 22.6; in its third round, at 4000 x 4,
+    // 32.9 against 23.6. The 8 x 4 tile holds 19456 sites at a time: 200 x 200 52.6 against 62.6 with 32 x 8 tiles,
+    // 16384 x 4 74.2 against 60.6 with 32 x 4. Beyond, 32 x 8 (2048^2 2170, 32 x 4 2540), a tube's 4 rows 32 x 4.
+    if (sites <= 9728) return V_RP8x4;
+    if (sites <= kF64SmallSites) return V_RP16x4;
+    return c->ny <= 4 ? V_T32x4 : V_T32x16;
   }
   // FP32 storage, times per step on a GB300 (us). Small grids are latency-bound: four lanes per node win up to
   // a few thousand sites (400 x 4: 10.3 against 16.4 with tiles; 2000 x 4: 14.4 against 16.4).

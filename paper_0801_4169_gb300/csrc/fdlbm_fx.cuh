@@ -134,6 +134,15 @@ FX_HD u64 shr_clamped(u64 v, int s) {
 }
 // v 2^-s rounded, |v| < 2^62, s in 0..63
 FX_HD s64 shr_round(s64 v, int s) { return (v + (s64)((1ull << s) >> 1)) >> s; }
+FX_HD s64 shl64(s64 v, int s) {  // 0 for s >= 64
+#ifdef __CUDA_ARCH__
+  s64 r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+  return r;
+#else
+  return s < 64 ? (s64)((u64)v << s) : 0;
+#endif
+}
 FX_HD unsigned shl_clamped(unsigned v, int s) {  // 0 for s >= 32
 #ifdef __CUDA_ARCH__
   unsigned r;

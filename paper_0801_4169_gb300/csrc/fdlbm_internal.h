@@ -116,8 +116,9 @@ inline void variant_tile(int v, int* tw, int* th) {
 // Launch configuration of the fused step: tile of TW x TH nodes per CTA, registers capped at 128
 // per thread (2-4 CTAs per SM). Phase 1 computes the moments of the tile and its 1-node ring,
 // (TW+2)(TH+2) - 4 nodes, in rounds of one node per thread. Which shape is fastest depends on the precision
-// and the grid, and the autotuner measures it.
-// V_RP* are the ring-parallel variants (four lanes per node) for small grids; batches use the
+// and the grid, and the autotuner measures it. FP32 storage has all of these; FP64 storage serves them with
+// five shapes (fdlbm_step_f64.cu), and its two-launch variants are its fused step.
+// V_RP* are the variants for small grids (FP32 storage: ring-parallel, four lanes per node); batches use the
 // tile variants only (V_TILE_COUNT).
 // V_S* split the step in two launches: k_moments writes every node's moments once to the grid's
 // moment buffer, and the update pass stages them for its tile and ring instead of recomputing
@@ -142,6 +143,17 @@ inline bool variant_graph(int v) { return v == V_GRP8x4; }
 inline int variant_one_step(int v) {
   return v == V_PRP8x4 || v == V_GRP8x4 ? V_RP8x4 : v == V_PT32x16 ? V_T32x16 : v;
 }
+// Tile shape of a batch's variant: FP64 storage has two (fdlbm_step_f64.cu).
+inline void batch_tile(int prec, int v, int* tw, int* th) {
+  variant_tile(v, tw, th);
+  if (prec == FDLBM_FP64) {
+    *tw = 32;
+    *th = v == V_T32x4 ? 4 : 8;
+  }
+}
+
+// FP64 storage: grids up to this many sites run the small tiles whatever the variant (fdlbm_step_f64.cu).
+constexpr long long kF64SmallSites = 40960;
 constexpr int kPersistMaxSteps = 4096;
 constexpr int kGraphSteps = 32;  // launches per captured graph (even: a replay ends in its first buffer)
 // fdlbm_autotune times every variant over at least this many steps on grids of up to 262144 sites.
@@ -153,10 +165,8 @@ cudaError_t launch_step_f64(int variant, const void* f, void* fn, const Grid& g,
                             cudaStream_t s);
 cudaError_t launch_step_f32(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
                             cudaStream_t s);
-// The tile variants (< V_TILE_COUNT) for a y-periodic grid with ny <= the tile height
-// (fdlbm_step_wrap_f32.cu, fdlbm_step_wrap_f64.cu); launch_step picks them.
-cudaError_t launch_step_wrap_f64(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c,
-                                 unsigned* health, cudaStream_t s);
+// FP32 storage: the tile variants (< V_TILE_COUNT) for a y-periodic grid with ny <= the tile height
+// (fdlbm_step_wrap_f32.cu); launch_step picks them.
 cudaError_t launch_step_wrap_f32(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c,
                                  unsigned* health, cudaStream_t s);
 // FDLBM_FP32_STORE_DW (fdlbm_step_f32dw.cu): the FP32-storage step with the per-ring equilibrium
@@ -166,6 +176,7 @@ cudaError_t launch_step_f32dw(int variant, const void* f, void* fn, const Grid& 
                               cudaStream_t s);
 cudaError_t launch_batch_f64(int variant, const BatchMember* mem, int nmem, long long tiles, unsigned long long step,
                              const Coeffs& c, cudaStream_t s);
+cudaError_t prepare_batch_f64(int variant);  // opt-in to its shared memory, outside stream capture
 cudaError_t launch_batch_f32(int variant, const BatchMember* mem, int nmem, long long tiles, unsigned long long step,
                              const Coeffs& c, cudaStream_t s);
 cudaError_t launch_gather_health(const BatchMember* mem, int nmem, unsigned* out, cudaStream_t s);

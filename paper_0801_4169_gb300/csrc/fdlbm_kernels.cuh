@@ -1,7 +1,7 @@
 #pragma once
 // fdlbm_kernels.cuh -- sm_103a kernels of the FDLBM step (Gan, Xu, Zhang, Yu, Li, arXiv 0801.4169).
-// Included by fdlbm_step_f64.cu / fdlbm_step_f32.cu (one precision each, compiled in parallel),
-// fdlbm_step_wrap_*.cu (tiles that hold a periodic grid's height) and fdlbm_aux.cu (initial
+// Included by fdlbm_fx64.cuh (the FP64-storage step), fdlbm_step_f32.cu, fdlbm_step_f32dw.cu,
+// fdlbm_step_wrap_f32.cu (tiles that hold a periodic grid's height) and fdlbm_aux.cu (initial
 // condition, boundary, moment and copy kernels).
 //
 // One fused kernel per time step computes, for every interior node of its tile:
@@ -446,18 +446,6 @@ __device__ __forceinline__ Mom node_moments(const float* __restrict__ f, long lo
   return fix_node_moments<true>(x, emax);
 }
 
-// One ring of a node (ring-parallel kernel, FP64 storage): S, X, Y of ring k, and f_0 (read by
-// every lane).
-template <bool COH = false>
-__device__ __forceinline__ void ring_of_node(const double* __restrict__ f, long long plane, long long off, int k,
-                                             double& f0, double& S, double& X, double& Y) {
-  double g[8];
-#pragma unroll
-  for (int d = 0; d < 8; ++d) g[d] = ldc<COH>(f + (long long)(1 + 8 * k + d) * plane + off);
-  f0 = ldc<COH>(f + off);
-  ring_sums(g, S, X, Y);
-}
-
 // (n, ux, uy, T, P) from the sums; T = (sum |v|^2 f)/(2n) - |u|^2/2  (Eq. 5 with P = nT). JS is
 // the unit of jx, jy in the sums: 1 for the FP64 sums, 100 for the fixed-point ones (hundredths,
 // with the energy sum in units of 1/JS^2).
@@ -489,39 +477,9 @@ __device__ __forceinline__ Macro node_macro(const float* __restrict__ f, long lo
   return to_macro<100>(node_moments<COH>(f, plane, off, c));
 }
 
-// Ring-parallel kernel: the macros of the quad's node, lane r of the quad (r = 0..3) summing ring
-// r. Every lane ends with the same values, bit for bit those of node_macro. All four lanes must
-// call it together.
-template <bool COH = false>
-__device__ __forceinline__ Macro quad_macro(const double* __restrict__ f, long long plane, long long off, int r,
-                                            const Coeffs& c) {
-  const unsigned ALL = 0xffffffffu;
-  double f0, S, X, Y;
-  ring_of_node<COH>(f, plane, off, r, f0, S, X, Y);
-  Mom m;
-  // n = ((f_0 + S_0) + S_1) + (S_2 + S_3), the tree of combine_rings
-  const double pn = (r == 0) ? f0 + S : S;
-  const double n2 = pn + __shfl_xor_sync(ALL, pn, 1);
-  m.n = n2 + __shfl_xor_sync(ALL, n2, 2);
-  // stage 1 (lanes r, r^1): j pair = fma(v_e, X_e, v_o X_o). The even lane sends its X (Y, S),
-  // the odd lane its product v X; each then forms the pair from identical operands.
-  const bool even = (r & 1) == 0;
-  const double prodx = c.v[r] * X, prody = c.v[r] * Y, prode = c.v2[r] * S;
-  const double o_x = __shfl_xor_sync(ALL, even ? X : prodx, 1);
-  const double o_y = __shfl_xor_sync(ALL, even ? Y : prody, 1);
-  const double o_e = __shfl_xor_sync(ALL, even ? S : prode, 1);
-  const int re = r & 2;  // the even lane of the pair
-  const double jx2 = even ? fma(c.v[re], X, o_x) : fma(c.v[re], o_x, prodx);
-  const double jy2 = even ? fma(c.v[re], Y, o_y) : fma(c.v[re], o_y, prody);
-  const double e22 = even ? fma(c.v2[re], S, o_e) : fma(c.v2[re], o_e, prode);
-  // stage 2 (pairs 01 and 23): commutative sums, equal in all four lanes
-  m.jx = jx2 + __shfl_xor_sync(ALL, jx2, 2);
-  m.jy = jy2 + __shfl_xor_sync(ALL, jy2, 2);
-  m.e2 = e22 + __shfl_xor_sync(ALL, e22, 2);
-  return to_macro<1>(m);
-}
-// FP32 storage: each lane forms its ring's exact sums, the quad adds the integers (exact, so in
-// any order) and exchanges the four S_k, and every lane finishes as node_moments does.
+// Ring-parallel kernel: the macros of the quad's node, bit for bit those of node_macro. Each lane forms its
+// ring's exact sums, the quad adds the integers (exact, so in any order) and exchanges the four S_k, and every
+// lane finishes as node_moments does. All four lanes call it together.
 template <bool COH = false>
 __device__ __forceinline__ Macro quad_macro(const float* __restrict__ f, long long plane, long long off, int r,
                                             const Coeffs& c) {
@@ -945,17 +903,6 @@ __device__ __forceinline__ S stencil_dir(const S* __restrict__ p, int pitch, con
 template <typename S>
 struct StencilConsts;
 template <>
-struct StencilConsts<double> {
-  __device__ static double W1(const Coeffs& c, int a, int k, int l) { return c.W1[a][k][l]; }
-  __device__ static double Wm1(const Coeffs& c, int a, int k, int l) { return c.Wm1[a][k][l]; }
-  __device__ static double D(const Coeffs& c, int a, int k, int l) { return c.D[a][k][l]; }
-  __device__ static double C2(const Coeffs& c, int k, int l) { return c.C2[k][l]; }
-  __device__ static double r(const Coeffs& c) { return c.r; }
-  __device__ static double kx(const Coeffs& c) { return c.kx; }
-  __device__ static double ky(const Coeffs& c) { return c.ky; }
-  __device__ static double lam(const Coeffs& c) { return c.lam; }
-};
-template <>
 struct StencilConsts<float> {
   __device__ static float W1(const Coeffs& c, int a, int k, int l) { return c.fW1[a][k][l]; }
   __device__ static float Wm1(const Coeffs& c, int a, int k, int l) { return c.fWm1[a][k][l]; }
@@ -967,12 +914,12 @@ struct StencilConsts<float> {
   __device__ static float lam(const Coeffs& c) { return c.flam; }
 };
 
-// Update of all 33 velocities at one interior node, given its moments and nu_x, nu_y. ES is the
-// equilibrium's site constants: EqSite, or EqSiteDW for the double-word variant (S = float).
-template <typename S, typename ES = EqSite, bool COH = false>
+// Update of ring K's 8 velocities at one interior node with the double-word equilibrium, from the node's site
+// constants and nu_x, nu_y.
+template <typename S, bool COH = false>
 __device__ __forceinline__ void update_ring(int K, const S* __restrict__ f, S* __restrict__ fn, const Grid& g,
                                             const Coeffs& c, long long off, int gx, int gy, const GhostOwn& go,
-                                            const ES& e, S w0base, S nux, S nuy) {
+                                            const EqSiteDW& e, S w0base, S nux, S nuy) {
   using SC = StencilConsts<S>;
   RingW<S> w;
 #pragma unroll
@@ -993,47 +940,25 @@ __device__ __forceinline__ void update_ring(int K, const S* __restrict__ f, S* _
   // All 8 directions of the ring are computed before any store, so the ring is one basic block
   // the compiler can interleave (the ghost-copy branch comes once per ring, not per velocity).
   S out[8];
-  if constexpr (std::is_same<ES, EqSiteDW>::value) {
-    S fe[8];
-    const EqRingDW er = eq_ring_dw(e, K, c);
-    eq_pair_dw(er, e.p[0], e.x[0], fe[7], fe[3]);
-    eq_pair_dw(er, e.p[1], e.x[1], fe[0], fe[4]);
-    eq_pair_dw(er, e.p[2], e.x[2], fe[1], fe[5]);
-    eq_pair_dw(er, e.p[3], e.x[3], fe[2], fe[6]);
+  S fe[8];
+  const EqRingDW er = eq_ring_dw(e, K, c);
+  eq_pair_dw(er, e.p[0], e.x[0], fe[7], fe[3]);
+  eq_pair_dw(er, e.p[1], e.x[1], fe[0], fe[4]);
+  eq_pair_dw(er, e.p[2], e.x[2], fe[1], fe[5]);
+  eq_pair_dw(er, e.p[3], e.x[3], fe[2], fe[6]);
 #pragma unroll
-    for (int d = 0; d < 8; ++d) {
-      const S* p = fq + (long long)(1 + 8 * K + d) * g.plane;
-      switch (d) {
-        case 0: out[0] = stencil_dir<S, 0, COH>(p, g.pitch, w, fe[0]); break;
-        case 1: out[1] = stencil_dir<S, 1, COH>(p, g.pitch, w, fe[1]); break;
-        case 2: out[2] = stencil_dir<S, 2, COH>(p, g.pitch, w, fe[2]); break;
-        case 3: out[3] = stencil_dir<S, 3, COH>(p, g.pitch, w, fe[3]); break;
-        case 4: out[4] = stencil_dir<S, 4, COH>(p, g.pitch, w, fe[4]); break;
-        case 5: out[5] = stencil_dir<S, 5, COH>(p, g.pitch, w, fe[5]); break;
-        case 6: out[6] = stencil_dir<S, 6, COH>(p, g.pitch, w, fe[6]); break;
-        default: out[7] = stencil_dir<S, 7, COH>(p, g.pitch, w, fe[7]); break;
-      }
+  for (int d = 0; d < 8; ++d) {
+    const S* p = fq + (long long)(1 + 8 * K + d) * g.plane;
+    switch (d) {
+      case 0: out[0] = stencil_dir<S, 0, COH>(p, g.pitch, w, fe[0]); break;
+      case 1: out[1] = stencil_dir<S, 1, COH>(p, g.pitch, w, fe[1]); break;
+      case 2: out[2] = stencil_dir<S, 2, COH>(p, g.pitch, w, fe[2]); break;
+      case 3: out[3] = stencil_dir<S, 3, COH>(p, g.pitch, w, fe[3]); break;
+      case 4: out[4] = stencil_dir<S, 4, COH>(p, g.pitch, w, fe[4]); break;
+      case 5: out[5] = stencil_dir<S, 5, COH>(p, g.pitch, w, fe[5]); break;
+      case 6: out[6] = stencil_dir<S, 6, COH>(p, g.pitch, w, fe[6]); break;
+      default: out[7] = stencil_dir<S, 7, COH>(p, g.pitch, w, fe[7]); break;
     }
-  } else {
-    static_assert(std::is_same<S, double>::value, "FP32 storage takes its f_eq from feq_ring");
-    const EqRing er = eq_ring(e, K, c);
-    S fp, fm;
-    // pair (d7: 0 deg, d3: 180 deg), projection p_x
-    eq_pair(er, e.p[0], e.x[0], fp, fm);
-    out[7] = stencil_dir<S, 7, COH>(fq + (long long)(1 + 8 * K + 7) * g.plane, g.pitch, w, fp);
-    out[3] = stencil_dir<S, 3, COH>(fq + (long long)(1 + 8 * K + 3) * g.plane, g.pitch, w, fm);
-    // pair (d0: 45 deg, d4: 225 deg), projection s(p_x + p_y)
-    eq_pair(er, e.p[1], e.x[1], fp, fm);
-    out[0] = stencil_dir<S, 0, COH>(fq + (long long)(1 + 8 * K + 0) * g.plane, g.pitch, w, fp);
-    out[4] = stencil_dir<S, 4, COH>(fq + (long long)(1 + 8 * K + 4) * g.plane, g.pitch, w, fm);
-    // pair (d1: 90 deg, d5: 270 deg), projection p_y
-    eq_pair(er, e.p[2], e.x[2], fp, fm);
-    out[1] = stencil_dir<S, 1, COH>(fq + (long long)(1 + 8 * K + 1) * g.plane, g.pitch, w, fp);
-    out[5] = stencil_dir<S, 5, COH>(fq + (long long)(1 + 8 * K + 5) * g.plane, g.pitch, w, fm);
-    // pair (d2: 135 deg, d6: 315 deg), projection s(p_y - p_x)
-    eq_pair(er, e.p[3], e.x[3], fp, fm);
-    out[2] = stencil_dir<S, 2, COH>(fq + (long long)(1 + 8 * K + 2) * g.plane, g.pitch, w, fp);
-    out[6] = stencil_dir<S, 6, COH>(fq + (long long)(1 + 8 * K + 6) * g.plane, g.pitch, w, fm);
   }
   store_ring<S>(fn, g, gx, gy, go, K, out);
 }
@@ -1298,7 +1223,7 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
   } else {
   const bool wrap = WRAPY && y0 == 0 && g.ny <= TH && g.bc[2] == BC_PERIODIC && g.bc[3] == BC_PERIODIC;
   const int nslot = wrap ? SW * g.ny : SW * SH;  // with wrap: local rows 1..ny only
-  constexpr int SLOTS = DW || std::is_same<S, double>::value ? NSLOT : 1;
+  constexpr int SLOTS = DW ? NSLOT : 1;
 #pragma unroll SLOTS
   for (int k = 0; k < NSLOT; ++k) {
     const int idx = tid + k * NT;
@@ -1350,27 +1275,24 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
       snuy = (S)0.5 * thy * aky * ((S)1 - aky);
     }
     const S w0base = ((S)1 - SC::r(c)) - (S)2 * (snux + snuy);
-    constexpr bool FXQ = std::is_same<S, float>::value && !DW;
-    using ES = typename std::conditional<DW, EqSiteDW, typename std::conditional<FXQ, FeqNode, EqSite>::type>::type;
-    ES e;
-    double snF = 0.0;
-    if constexpr (DW) e = eq_site_dw(n, ux, uy, T, c);
-    else if constexpr (FXQ) e = feq_node<S>(n, ux, uy, T, c);
-    else e = eq_site(n, ux, uy, T, c);
     const long long off = (long long)(gy + NG) * g.pitch + (gx + NG);
     const GhostOwn go = ghost_own(g, gx, gy);
     // rest velocity: f_eq = n F_0 A0; c = 0 on both axes (line IV only)
-    if constexpr (!FXQ) {
-      S rfeq;
-      if constexpr (DW) rfeq = e.rest;
-      else rfeq = to_s<S>(e.rest);
+    auto rest = [&](S rfeq) {
       const S* p = f + off;
       S acc = fma(w0base, ldc<COH>(p), rfeq);
       acc = fma(snux, ldc<COH>(p + 1) + ldc<COH>(p - 1), acc);
       acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
       store_node<S, 0>(fn, g, gx, gy, go, acc);
-    }
-    if constexpr (std::is_same<S, float>::value && !DW) {
+    };
+    if constexpr (DW) {
+      const EqSiteDW e = eq_site_dw(n, ux, uy, T, c);
+      rest(e.rest);
+#pragma unroll
+      for (int K = 0; K < 4; ++K) update_ring<S, COH>(K, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+    } else {
+      const FeqNode e = feq_node<S>(n, ux, uy, T, c);
+      double snF = 0.0;
 #pragma unroll 1
       for (int K = 0; K < 4; ++K) {
         const double nF = ring_weight<false>(e, K, c);
@@ -1379,16 +1301,7 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
         feq_ring(e, K, nF, c, n, ux, uy, T, fe);
         ring_stencil<S, COH>(K, f, fn, g, c, off, gx, gy, go, fe, w0base, snux, snuy);
       }
-      const S* p = f + off;
-      S acc = fma(w0base, ldc<COH>(p), feq_rest(e, n, snF, c));
-      acc = fma(snux, ldc<COH>(p + 1) + ldc<COH>(p - 1), acc);
-      acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
-      store_node<S, 0>(fn, g, gx, gy, go, acc);
-    } else {
-      update_ring<S, ES, COH>(0, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-      update_ring<S, ES, COH>(1, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-      update_ring<S, ES, COH>(2, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
-      update_ring<S, ES, COH>(3, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      rest(feq_rest(e, n, snF, c));
     }
   }
   }
@@ -1453,9 +1366,8 @@ __global__ void __launch_bounds__(BX * BY, MINB) k_step_batch(const BatchMember*
 
 // Ring-parallel step for small grids, where one thread per node leaves the GPU's FP64 pipes
 // waiting on long dependency chains. Four lanes share a node, lane r holding velocity ring r:
-// - Moments (quad_macro): each lane sums its ring. With FP64 storage two shuffle stages combine
-//   the rings in the same pairwise tree as node_moments; with FP32 storage the quad adds the exact
-//   integer sums. Either way the moments are bit for bit those of k_step.
+// - Moments (quad_macro): each lane sums its ring and the quad adds the exact integer sums, so the moments
+//   are bit for bit those of k_step.
 // - Update: all four lanes evaluate the node's constants (switch, weights, f_eq site terms).
 //   That costs no extra issue slots: it is one warp instruction whether one lane or four use it.
 //   Each lane then updates its own 8 velocities, and lane 0 also the rest velocity.
@@ -1531,24 +1443,18 @@ __device__ __forceinline__ void rp_tile(const S* __restrict__ f, S* __restrict__
       acc = fma(snuy, ldc<COH>(p + g.pitch) + ldc<COH>(p - g.pitch), acc);
       store_node<S, 0>(fn, g, gx, gy, go, acc);
     };
-    if constexpr (std::is_same<S, float>::value) {
-      const FeqNode e = feq_node<S>(n, ux, uy, T, c);
-      double nF = 0.0, snF = 0.0;
+    const FeqNode e = feq_node<S>(n, ux, uy, T, c);
+    double nF = 0.0, snF = 0.0;
 #pragma unroll
-      for (int K = 0; K < 4; ++K) {
-        const double w = ring_weight<false>(e, K, c);
-        snF += w;
-        if (K == r) nF = w;
-      }
-      if (r == 0) rest(feq_rest(e, n, snF, c));
-      S fe[8];
-      feq_ring(e, r, nF, c, n, ux, uy, T, fe);
-      ring_stencil<S, COH>(r, f, fn, g, c, off, gx, gy, go, fe, w0base, snux, snuy);
-    } else {
-      const EqSite e = eq_site(n, ux, uy, T, c);
-      if (r == 0) rest(e.rest);
-      update_ring<S, EqSite, COH>(r, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+    for (int K = 0; K < 4; ++K) {
+      const double w = ring_weight<false>(e, K, c);
+      snF += w;
+      if (K == r) nF = w;
     }
+    if (r == 0) rest(feq_rest(e, n, snF, c));
+    S fe[8];
+    feq_ring(e, r, nF, c, n, ux, uy, T, fe);
+    ring_stencil<S, COH>(r, f, fn, g, c, off, gx, gy, go, fe, w0base, snux, snuy);
   }
   if (bits) atomicOr(health, bits);
 }
@@ -1774,23 +1680,16 @@ cudaError_t launch_step_v(int variant, const void* f, void* fn, const Grid& g, c
     case V_T32x16: return launch_step_t<S, 32, 8, 2, 2, false, true, DW>(f, fn, g, c, health, s);
     case V_T16x4: return launch_step_t<S, 16, 4, 1, 1, false, false, DW>(f, fn, g, c, health, s);
     case V_T64x8: return launch_step_t<S, 64, 4, 2, 2, false, true, DW>(f, fn, g, c, health, s);
-    case V_T32x32:
-      if constexpr (std::is_same<S, float>::value) return launch_step_t<S, 32, 4, 1, 6, false, true, DW>(f, fn, g, c, health, s);
-      else return launch_step_t<S, 32, 8, 4, 2>(f, fn, g, c, health, s);
-    case V_T32x24:
-      // FP32 storage: a staged 32 x 8 tile at <= 85 registers for 3 CTAs per SM (24 warps); FP64
-      // storage keeps the 32 x 24 tile of 128 threads
-      if constexpr (std::is_same<S, float>::value) return launch_step_t<S, 32, 8, 1, 3, false, true, DW>(f, fn, g, c, health, s);
-      else return launch_step_t<S, 32, 4, 6, 4>(f, fn, g, c, health, s);
-    case V_T32x28:
-      if constexpr (std::is_same<S, float>::value) return launch_step_t<S, 32, 8, 1, 4, false, true, DW>(f, fn, g, c, health, s);
-      else return launch_step_t<S, 32, 4, 7, 4>(f, fn, g, c, health, s);
+    case V_T32x32: return launch_step_t<S, 32, 4, 1, 6, false, true, DW>(f, fn, g, c, health, s);
+    // a staged 32 x 8 tile at <= 85 registers for 3 CTAs per SM (24 warps)
+    case V_T32x24: return launch_step_t<S, 32, 8, 1, 3, false, true, DW>(f, fn, g, c, health, s);
+    case V_T32x28: return launch_step_t<S, 32, 8, 1, 4, false, true, DW>(f, fn, g, c, health, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 // The tile variants for a grid whose whole y-periodic height fits in one tile (step_tile WRAPY):
-// instantiated in their own translation units, fdlbm_step_wrap_*.cu.
+// instantiated in their own translation unit, fdlbm_step_wrap_f32.cu.
 template <typename S>
 cudaError_t launch_step_wrap_v(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c,
                                unsigned* health, cudaStream_t s) {
