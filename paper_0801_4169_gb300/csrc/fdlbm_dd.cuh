@@ -64,6 +64,25 @@ __device__ __forceinline__ dd_t sqr(dd_t a) {
   p.lo = __fma_rn(2.0 * a.hi, a.lo, p.lo);
   return quick_two_sum(p.hi, p.lo);
 }
+// A sum of products a b kept as s + e, normalized once at the end: 12 operations a product, where mul and add
+// take 18. s is the FP64 sum of the products' leading parts, e collects what its additions and the products
+// leave over, so the error stays a few units of 2^-106 of the largest partial sum, as with mul and add.
+struct dot {
+  double s, e;
+};
+__device__ __forceinline__ dot dot_of(dd_t a) { return {a.hi, a.lo}; }
+__device__ __forceinline__ dot dot_start(dd_t a, dd_t b) {
+  const double p = __dmul_rn(a.hi, b.hi);
+  return {p, __fma_rn(a.hi, b.lo, __fma_rn(a.lo, b.hi, __fma_rn(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ void dot_add(dot& d, dd_t a, dd_t b) {
+  const double p = __dmul_rn(a.hi, b.hi);
+  const double q = __fma_rn(a.hi, b.hi, -p);
+  const dd_t t = two_sum(d.s, p);
+  d.s = t.hi;
+  d.e = __dadd_rn(__fma_rn(a.hi, b.lo, __fma_rn(a.lo, b.hi, d.e)), __dadd_rn(q, t.lo));
+}
+__device__ __forceinline__ dd_t dot_end(dot d) { return quick_two_sum(d.s, d.e); }
 // Multiplication by a power of two is exact.
 __device__ __forceinline__ dd_t scale2(dd_t a, double p2) { return {a.hi * p2, a.lo * p2}; }
 
@@ -85,7 +104,7 @@ __device__ __forceinline__ dd_t div(dd_t a, double b) { return div(a, make(b)); 
 
 // 1/sqrt(a), a > 0: FP64 estimate refined by one Newton step, y = y0 + y0 (1 - a y0^2) / 2.
 __device__ __forceinline__ dd_t rsqrt(dd_t a) {
-  const double y0 = 1.0 / ::sqrt(a.hi);
+  const double y0 = ::rsqrt(a.hi);
   const dd_t e = sub(make(1.0), mul(mul(a, y0), y0));
   return quick_two_sum(y0, __dmul_rn(0.5 * e.hi, y0));
 }
@@ -110,9 +129,17 @@ __device__ __forceinline__ cdd cmul(cdd a, cdd b) {
   return {sub(mul(a.re, b.re), mul(a.im, b.im)), add(mul(a.re, b.im), mul(a.im, b.re))};
 }
 __device__ __forceinline__ cdd cmul(cdd a, dd_t b) { return {mul(a.re, b), mul(a.im, b)}; }
-// conj(a) * b
-__device__ __forceinline__ cdd cmulc(cdd a, cdd b) {
-  return {add(mul(a.re, b.re), mul(a.im, b.im)), sub(mul(a.re, b.im), mul(a.im, b.re))};
+// z + a b, z as its two sums
+__device__ __forceinline__ void cdot_add(dot& re, dot& im, cdd a, cdd b) {
+  dot_add(re, a.re, b.re);
+  dot_add(im, a.re, b.im);
+  dot_add(re, neg(a.im), b.im);
+  dot_add(im, a.im, b.re);
+}
+__device__ __forceinline__ cdd csubmul(cdd z, cdd a, cdd b) {  // z - a b
+  dot re = dot_of(z.re), im = dot_of(z.im);
+  cdot_add(re, im, {neg(a.re), neg(a.im)}, b);
+  return {dot_end(re), dot_end(im)};
 }
 __device__ __forceinline__ dd_t cabs2(cdd a) { return add(sqr(a.re), sqr(a.im)); }
 // Principal square root: with r = |z|, t = sqrt((r + |x|)/2), the root is (t, y/2t) for x >= 0

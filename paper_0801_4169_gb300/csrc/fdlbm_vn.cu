@@ -7,16 +7,18 @@
 //      i), column factors d(n, T, u_x, u_y) / d f_j (lane j), and the diagonal symbol of Eq. 17.
 //   2. Householder reduction to upper Hessenberg form (lanes over columns, then over rows).
 //   3. Single-shift QR sweeps with Givens rotations restricted to the active block (eigenvalues
-//      only). The rotation of row pair k is computed, the column rotation k-1 is applied right
-//      after it (the two touch different data), so a sweep stores no rotations. Shifts are
+//      only). The rotation of row pair k is computed and applied together with the column
+//      rotation k-1 (rotate_both), so a sweep stores no rotations. Shifts are
 //      Wilkinson's, in double-double: an FP64 shift stalls into linear convergence on the
 //      near-double eigenvalues that coinciding stencil symbols produce. A 1 x 1 or 2 x 2 block
 //      that splits off is solved directly.
-// Scalar steps (a rotation's parameters, a shift) are computed by every lane alike, so no lane
-// waits on another beyond __syncwarp.
+// A rotation's squares and products are spread over four lanes; a shift is computed by every lane alike.
 //
-// FP64 issues at ~2 instructions/clk/SM on this part, so the kernel is bound by the FP64 pipe;
-// six single-warp CTAs share an SM (6 x 35 KB of shared memory).
+// FP64 issues at ~2 instructions/clk/SM on this part, so the kernel is bound by the FP64 pipe, and what counts is
+// the number of warp instructions; six single-warp CTAs share an SM (6 x 35 KB of shared memory). The Sec. 4
+// sweep (22 x 256 spectra): 226 ms with a normalized double-double operation for every product and sum, rows
+// and columns rotated one after the other; 149 ms with sums of products normalized once (dot) and one list for
+// both; 146 with a component a lane.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -123,83 +125,91 @@ __device__ __forceinline__ double l1_hi(const cdd& z) { return fabs(z.re.hi) + f
 // square root. Applied from the left to rows k, k+1, and as U^H from the right to columns k, k+1.
 struct Rot {
   cdd a, b;
+  dd_t r;
 };
-__device__ Rot givens(const cdd& x, const cdd& y) {
-  const dd_t r2 = dd::add(dd::cabs2(x), dd::cabs2(y));
+// Lane parts: lane & 3 squares one of x.re, x.im, y.re, y.im and scales it; every lane ends with the same
+// rotation (the butterfly's additions are commutative bit for bit).
+__device__ Rot givens(const cdd& x, const cdd& y, int lane) {
+  const unsigned ALL = 0xffffffffu;
+  const dd_t u = (lane & 1) ? x.im : x.re, w = (lane & 1) ? y.im : y.re, v = (lane & 2) ? w : u;
+  dd_t r2 = dd::sqr(v);
+#pragma unroll
+  for (int m = 1; m <= 2; m <<= 1)
+    r2 = dd::add(r2, {__shfl_xor_sync(ALL, r2.hi, m), __shfl_xor_sync(ALL, r2.lo, m)});
   Rot g;
   if (r2.hi == 0.0) {
     g.a = {dd::make(1.0), dd::make(0.0)};
     g.b = {dd::make(0.0), dd::make(0.0)};
+    g.r = dd::make(0.0);
     return g;
   }
-  const dd_t rinv = dd::rsqrt(r2);
-  g.a = dd::cmul(dd::cconj(x), rinv);
-  g.b = dd::cmul(dd::cconj(y), rinv);
+  const dd_t rinv = dd::rsqrt(r2), p = dd::mul(v, rinv);
+  auto part = [&](int l) { return dd_t{__shfl_sync(ALL, p.hi, l), __shfl_sync(ALL, p.lo, l)}; };
+  g.a = dd::cconj({part(0), part(1)});
+  g.b = dd::cconj({part(2), part(3)});
+  g.r = dd::mul(r2, rinv);
   return g;
 }
-// One output element of a rotation, one lane each: lane parity picks the output row (left
-// product: new_k = a X + b Y, new_k+1 = -conj(b) X + conj(a) Y) or column (right product by U^H:
-// new_k = conj(a) P + conj(b) Q, new_k+1 = -b P + a Q). Both lanes of a pair read the same two
-// inputs, so the warp reads everything before anyone writes.
-__device__ __forceinline__ void rot_coeffs_left(const Rot& g, bool second, cdd* al, cdd* be) {
-  if (!second) {
-    *al = g.a;
-    *be = g.b;
-  } else {
-    *al = dd::cconj(g.b);
-    al->re = dd::neg(al->re);
-    al->im = dd::neg(al->im);
-    *be = dd::cconj(g.a);
-  }
+// One component of one output element of a rotation a lane: lane & 1 picks the output row (left product:
+// new_k = a X + b Y, new_k+1 = -conj(b) X + conj(a) Y) or column (right product by U^H: new_k = conj(a) P +
+// conj(b) Q, new_k+1 = -b P + a Q), lane & 2 the imaginary part. A component is c0 X_0 + c1 X_1 + c2 Y_0 + c3 Y_1
+// with X_0 the part of its own kind and X_1 the other. The four lanes of an element read the same two inputs, so
+// the warp reads everything before anyone writes. Eight elements a pass (43 FP64 instructions): with both
+// components on a lane, 16 elements a pass of 86, narrow blocks left half the lanes idle.
+struct Coef {
+  dd_t c[4];
+};
+__device__ __forceinline__ Coef rot_coeffs(cdd al, cdd be, bool im) {
+  return {{al.re, im ? al.im : dd::neg(al.im), be.re, im ? be.im : dd::neg(be.im)}};
 }
-__device__ __forceinline__ void rot_coeffs_right(const Rot& g, bool second, cdd* al, cdd* be) {
-  if (!second) {
-    *al = dd::cconj(g.a);
-    *be = dd::cconj(g.b);
-  } else {
-    *al = {dd::neg(g.b.re), dd::neg(g.b.im)};
-    *be = g.a;
-  }
+__device__ __forceinline__ Coef coeffs_left(const Rot& g, int lane) {
+  const cdd nb = {dd::neg(g.b.re), g.b.im};  // -conj(b)
+  return lane & 1 ? rot_coeffs(nb, dd::cconj(g.a), lane & 2) : rot_coeffs(g.a, g.b, lane & 2);
 }
-// rows (k, k+1) over columns j0 .. j1
-__device__ __forceinline__ void rotate_rows(VnShared& S, const Rot& g, int k, int j0, int j1, int lane) {
-  cdd al, be;
-  rot_coeffs_left(g, lane & 1, &al, &be);
-  const int row = k + (lane & 1);
-  for (int base = j0; base <= j1; base += 16) {
-    const int j = base + (lane >> 1);
-    const bool act = j <= j1;
-    cdd X, Y;
+__device__ __forceinline__ Coef coeffs_right(const Rot& g, int lane) {
+  const cdd nb = {dd::neg(g.b.re), dd::neg(g.b.im)};
+  return lane & 1 ? rot_coeffs(nb, g.a, lane & 2) : rot_coeffs(dd::cconj(g.a), dd::cconj(g.b), lane & 2);
+}
+// Rotation g of rows (k, k+1) over columns k .. hi, and, unless k = lo, the rotation prev of columns (k-1, k) over
+// rows lo .. k, in one list of hi - lo + 1 elements. The two meet in (k, k) only, which g makes r: its column
+// rotation takes r in place of the entry. (k+1, k) becomes zero, exactly. rows 0 (no g) leaves the columns
+// (k-1, k) over rows lo .. k.
+__device__ __forceinline__ void rotate_both(VnShared& S, const Rot& g, const Rot& prev, int k, int lo, int hi, int rows,
+                                            int lane) {
+  const Coef L = coeffs_left(g, lane), R = coeffs_right(prev, lane);
+  double2* const part = lane & 2 ? S.im : S.re;
+  const double2* const other = lane & 2 ? S.re : S.im;
+  const int all = rows + (k > lo ? k - lo + 1 : 0);
+  for (int base = 0; base < all; base += 8) {
+    const int e = base + (lane >> 2), i = lo + e - rows;
+    const bool act = e < all, left = e < rows;
+    const int x = left ? k * N + k + 1 + e : i * N + k - 1, y = left ? x + N : x + 1;
+    dd_t X0, X1, Y0, Y1;
     if (act) {
-      X = ldA(S, k, j);
-      Y = ldA(S, k + 1, j);
+      X0 = ldd(part[x]);
+      X1 = ldd(other[x]);
+      Y0 = ldd(part[y]);
+      Y1 = ldd(other[y]);
+      if (rows != 0 && !left && i == k) {
+        X0 = X1 = dd::make(0.0);
+        Y0 = lane & 2 ? dd::make(0.0) : g.r;
+        Y1 = lane & 2 ? g.r : dd::make(0.0);
+      }
     }
     __syncwarp();
     if (act) {
-      cdd out = dd::cadd(dd::cmul(al, X), dd::cmul(be, Y));
-      if (row == k + 1 && j == k) out = cdd{dd::make(0.0), dd::make(0.0)};  // the zeroed entry, exactly
-      stA(S, row, j, out);
+      dd::dot d = dd::dot_start(left ? L.c[0] : R.c[0], X0);
+      dd::dot_add(d, left ? L.c[1] : R.c[1], X1);
+      dd::dot_add(d, left ? L.c[2] : R.c[2], Y0);
+      dd::dot_add(d, left ? L.c[3] : R.c[3], Y1);
+      part[lane & 1 ? y : x] = std2(dd::dot_end(d));
     }
-    __syncwarp();
   }
-}
-// columns (k, k+1) over rows i0 .. i1, by U^H from the right
-__device__ __forceinline__ void rotate_cols(VnShared& S, const Rot& g, int k, int i0, int i1, int lane) {
-  cdd al, be;
-  rot_coeffs_right(g, lane & 1, &al, &be);
-  const int col = k + (lane & 1);
-  for (int base = i0; base <= i1; base += 16) {
-    const int i = base + (lane >> 1);
-    const bool act = i <= i1;
-    cdd P, Qv;
-    if (act) {
-      P = ldA(S, i, k);
-      Qv = ldA(S, i, k + 1);
-    }
-    __syncwarp();
-    if (act) stA(S, i, col, dd::cadd(dd::cmul(P, al), dd::cmul(Qv, be)));
-    __syncwarp();
+  if (rows != 0 && lane == 0) {
+    stA(S, k + 1, k, cdd{dd::make(0.0), dd::make(0.0)});
+    if (k == lo) stA(S, k, k, cdd{g.r, dd::make(0.0)});
   }
+  __syncwarp();
 }
 
 __global__ void __launch_bounds__(32) k_vn(const fdlbm_vn_case* __restrict__ cases, double dx, double dy,
@@ -368,15 +378,15 @@ __global__ void __launch_bounds__(32) k_vn(const fdlbm_vn_case* __restrict__ cas
     // left: columns k+1 .. N-1 (lane l -> column k+1+l), A -= v (beta v^H A)
     if (lane < m) {
       const int j = k + 1 + lane;
-      cdd w = {dd::make(0.0), dd::make(0.0)};
+      dd::dot wr{0.0, 0.0}, wi{0.0, 0.0};
       for (int i = 0; i < m; ++i) {
         const cdd vi = {ldd(S.v[2 * i]), ldd(S.v[2 * i + 1])};
-        w = dd::cadd(w, dd::cmulc(vi, ldA(S, k + 1 + i, j)));
+        dd::cdot_add(wr, wi, dd::cconj(vi), ldA(S, k + 1 + i, j));
       }
-      w = dd::cmul(w, beta);
+      const cdd w = dd::cmul(cdd{dd::dot_end(wr), dd::dot_end(wi)}, beta);
       for (int i = 0; i < m; ++i) {
         const cdd vi = {ldd(S.v[2 * i]), ldd(S.v[2 * i + 1])};
-        stA(S, k + 1 + i, j, dd::csub(ldA(S, k + 1 + i, j), dd::cmul(vi, w)));
+        stA(S, k + 1 + i, j, dd::csubmul(ldA(S, k + 1 + i, j), vi, w));
       }
     }
     // column k becomes (alpha, 0, ..., 0) below the diagonal
@@ -386,15 +396,15 @@ __global__ void __launch_bounds__(32) k_vn(const fdlbm_vn_case* __restrict__ cas
     // column k+1+j, the dot product is a warp sum), so no lane runs a second pass alone.
     {
       const int i = lane;
-      cdd w = {dd::make(0.0), dd::make(0.0)};
+      dd::dot wr{0.0, 0.0}, wi{0.0, 0.0};
       for (int j = 0; j < m; ++j) {
         const cdd vj = {ldd(S.v[2 * j]), ldd(S.v[2 * j + 1])};
-        w = dd::cadd(w, dd::cmul(ldA(S, i, k + 1 + j), vj));
+        dd::cdot_add(wr, wi, ldA(S, i, k + 1 + j), vj);
       }
-      w = dd::cmul(w, beta);
+      const cdd w = dd::cmul(cdd{dd::dot_end(wr), dd::dot_end(wi)}, beta);
       for (int j = 0; j < m; ++j) {
         const cdd vj = {ldd(S.v[2 * j]), ldd(S.v[2 * j + 1])};
-        stA(S, i, k + 1 + j, dd::csub(ldA(S, i, k + 1 + j), dd::cmul(w, dd::cconj(vj))));
+        stA(S, i, k + 1 + j, dd::csubmul(ldA(S, i, k + 1 + j), w, dd::cconj(vj)));
       }
     }
     {
@@ -404,7 +414,7 @@ __global__ void __launch_bounds__(32) k_vn(const fdlbm_vn_case* __restrict__ cas
         t = dd::cmul(ldA(S, N - 1, k + 1 + lane), vl);
       }
       const cdd w = dd::cmul(cdd{warp_sum(t.re), warp_sum(t.im)}, beta);
-      if (lane < m) stA(S, N - 1, k + 1 + lane, dd::csub(ldA(S, N - 1, k + 1 + lane), dd::cmul(w, dd::cconj(vl))));
+      if (lane < m) stA(S, N - 1, k + 1 + lane, dd::csubmul(ldA(S, N - 1, k + 1 + lane), w, dd::cconj(vl)));
     }
     __syncwarp();
   }
@@ -469,15 +479,14 @@ __global__ void __launch_bounds__(32) k_vn(const fdlbm_vn_case* __restrict__ cas
     __syncwarp();
     for (int q = lo + lane; q <= hi; q += 32) stA(S, q, q, dd::csub(ldA(S, q, q), mu));
     __syncwarp();
-    Rot prev;
+    Rot prev{};
     for (int k = lo; k < hi; ++k) {
-      const Rot g = givens(ldA(S, k, k), ldA(S, k + 1, k));
+      const Rot g = givens(ldA(S, k, k), ldA(S, k + 1, k), lane);
       __syncwarp();
-      rotate_rows(S, g, k, k, hi, lane);                // left rotation of rows k, k+1
-      if (k > lo) rotate_cols(S, prev, k - 1, lo, k, lane);  // right rotation k-1 over rows lo..k
+      rotate_both(S, g, prev, k, lo, hi, hi - k, lane);
       prev = g;
     }
-    rotate_cols(S, prev, hi - 1, lo, hi, lane);
+    rotate_both(S, prev, prev, hi, lo, hi, 0, lane);  // the last columns
     for (int q = lo + lane; q <= hi; q += 32) stA(S, q, q, dd::cadd(ldA(S, q, q), mu));
     __syncwarp();
   }
