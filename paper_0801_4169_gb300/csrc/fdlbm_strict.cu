@@ -28,11 +28,23 @@
 //                          theta_a = lambda |((P+ - 2 P0) + P-) / ((P+ + 2 P0) + P-)| (Eq. 16),
 //                          P = n T at I+1, I, I-1 along alpha.
 //
-// It is the library's reference-grade path, not its fast one: one thread per node, no shared
-// memory, every division a division. Two launches per step: the moments of every node that the
-// update reads (the interior and the ghost layer next to each edge) into the moment buffer, then
-// the update of every interior node with the ghost copies it owns (periodic, zero-gradient,
-// mirror). Dirichlet ghosts, the initial condition and boundary segments take the same f_eq.
+// Two launches per step: the moments of every node that the update reads (the interior and the ghost layer
+// next to each edge) into the moment buffer, then the update of every interior node with the ghost copies it
+// owns (periodic, zero-gradient, mirror). Dirichlet ghosts, the initial condition and boundary segments take
+// the same f_eq.
+//
+// The step is bound by the FP64 pipe, and with every operation above taken as written for every node and
+// velocity, most of it were divisions (300 x 75: 434 us per step; 192 now). The same bits come from fewer operations:
+//   - c and what Eq. 17 forms from it alone depend on the velocity and the axis, not on the node: the host
+//     forms them once per launch, with the same operations; a negative component only changes signs;
+//   - opposite velocities have v.u of opposite sign and the same magnitude, so one set of quotients serves both;
+//   - a quotient by theta, 2 theta^2, 6 theta^3 or 24 theta^4 is a q1 = q0 + (a - b q0) y step from the correctly
+//     rounded y = 1/b, taken twice; by Markstein's theorem (IBM J. Res. Dev. 34, 1990) the second is the
+//     correctly rounded quotient. Operands outside 2^+-600 and b outside 2^+-210 take the division.
+// The update has one thread for each node and velocity ring, since a small grid has too few nodes to fill the
+// schedulers evenly.
+#include <cmath>
+
 #include "fdlbm_kernels.cuh"
 
 namespace fdlbm {
@@ -140,47 +152,89 @@ __device__ __forceinline__ bool mac_ok(const Mac& m) {
   return isfinite(m.n) && isfinite(m.ux) && isfinite(m.uy) && isfinite(m.T) && m.n > 0.0 && m.T > 0.0;
 }
 
-// Raw scheme parameters: the ratios are formed on the device, in the order above.
+// Scheme parameters and what the host forms from them, in the order above: F_k's numerator coefficients and
+// denominator, and c/2, (c c)/2, (c (1 - c c))/12 for axis a, ring k, l = 0 along the axis, 1 diagonal.
 struct Params {
-  double dt, tau, dr[2], lam;
+  double dt, dr[2], lam, r;
+  double w3[4], w2[4], w1[4], den[4];
+  double c1[2][4][2], c2[2][4][2], c3[2][4][2];
   int flags;
 };
 
-template <int QQ>
-__device__ __forceinline__ void update_one(const double* __restrict__ f, double* __restrict__ fn, const Grid& g,
-                                           const Params& p, long long off, int gx, int gy, const GhostOwn& go,
-                                           const Mac& m, const double (&F)[5], double r, const double (&sw)[2],
-                                           const double (&kap)[2]) {
-  double vx, vy;
-  vel(QQ, vx, vy);
-  const double fe = feq(QQ, m.n, m.ux, m.uy, m.T, F);
-  const double* fq = f + (long long)QQ * g.plane + off;
-  const double f0 = fq[0];
-  double acc = sub(f0, mul(r, sub(f0, fe)));
-#pragma unroll
-  for (int a = 0; a < 2; ++a) {
-    const long long st = a == 0 ? 1 : g.pitch;
-    const double fp1 = fq[st], fm1 = fq[-st], fp2 = fq[2 * st], fm2 = fq[-2 * st];
-    const double c = dvd(mul(a == 0 ? vx : vy, p.dt), p.dr[a]);
-    acc = sub(acc, mul(dvd(c, 2.0), sub(fp1, fm1)));
-    if (!(p.flags & F_NO_LW)) acc = add(acc, mul(dvd(mul(c, c), 2.0), add(sub(fp1, mul(2.0, f0)), fm1)));
-    if (!(p.flags & F_NO_DISP))
-      acc = add(acc, mul(dvd(mul(c, sub(1.0, mul(c, c))), 12.0),
-                         sub(add(sub(fp2, mul(2.0, fp1)), mul(2.0, fm1)), fm2)));
-    if (!(p.flags & F_NO_VISC)) {
-      const double ak = fabs(kap[a]);
-      acc = add(acc, mul(dvd(mul(mul(sw[a], ak), sub(1.0, ak)), 2.0), add(sub(fp1, mul(2.0, f0)), fm1)));
-    }
-  }
-  store_node<double, QQ>(fn, g, gx, gy, go, acc);
+__device__ __noinline__ double dvd_rare(double a, double b) { return dvd(a, b); }
+// a / b for b in 2^+-210, y = 1/b rounded to nearest
+__device__ __forceinline__ double dvd_by(double a, double b, double y) {
+  const unsigned ah = (unsigned)__double2hiint(a) & 0x7fffffffu;
+  if (__builtin_expect(ah - ((1023u - 600u) << 20) >= 1200u << 20, 0))
+    return (ah | (unsigned)__double2loint(a)) ? dvd_rare(a, b) : a;  // b > 0: a zero keeps its sign
+  const double q0 = mul(a, y);
+  const double q1 = __fma_rn(__fma_rn(-b, q0, a), y, q0);
+  return __fma_rn(__fma_rn(-b, q1, a), y, q1);
 }
 
-template <int... QS>
-__device__ __forceinline__ void update_all(const double* __restrict__ f, double* __restrict__ fn, const Grid& g,
-                                           const Params& p, long long off, int gx, int gy, const GhostOwn& go,
-                                           const Mac& m, const double (&F)[5], double r, const double (&sw)[2],
-                                           const double (&kap)[2]) {
-  (update_one<QS>(f, fn, g, p, off, gx, gy, go, m, F, r, sw, kap), ...);
+// What Eq. 10 shares between a node's velocities
+struct EqNode {
+  double t0, h, b[4], y[4];
+  bool near;  // theta in 2^+-50: dvd_by
+};
+__device__ __forceinline__ EqNode eq_node(double ux, double uy, double th) {
+  EqNode e;
+  const double u2 = add(mul(ux, ux), mul(uy, uy));
+  e.h = sub(1.0, dvd(u2, mul(2.0, th)));
+  e.t0 = add(e.h, dvd(mul(u2, u2), mul(mul(8.0, th), th)));
+  e.b[0] = th;
+  e.b[1] = mul(mul(2.0, th), th);
+  e.b[2] = mul(mul(mul(6.0, th), th), th);
+  e.b[3] = mul(mul(mul(mul(24.0, th), th), th), th);
+  const unsigned hi = (unsigned)__double2hiint(th);
+  e.near = hi - ((1023u - 50u) << 20) < 100u << 20;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) e.y[i] = e.near ? __drcp_rn(e.b[i]) : 0.0;
+  return e;
+}
+// The bracket of Eq. 10 for v.u = vu and for -vu
+__device__ __forceinline__ void brackets(const EqNode& e, double vu, double& plus, double& minus) {
+  const double p2 = mul(vu, vu), p3 = mul(p2, vu), p4 = mul(p3, vu);
+  double q1, q2, q3, q4;
+  if (__builtin_expect(e.near, 1)) {
+    q1 = dvd_by(vu, e.b[0], e.y[0]);
+    q2 = dvd_by(p2, e.b[1], e.y[1]);
+    q3 = dvd_by(p3, e.b[2], e.y[2]);
+    q4 = dvd_by(p4, e.b[3], e.y[3]);
+  } else {
+    q1 = dvd_rare(vu, e.b[0]);
+    q2 = dvd_rare(p2, e.b[1]);
+    q3 = dvd_rare(p3, e.b[2]);
+    q4 = dvd_rare(p4, e.b[3]);
+  }
+  const double t1 = mul(q1, e.h), t2 = mul(q2, e.h);
+  plus = add(add(add(add(e.t0, t1), t2), q3), q4);
+  minus = add(sub(add(sub(e.t0, t1), t2), q3), q4);
+}
+__device__ __forceinline__ double weight(const Params& p, int k, double th, double t2, double t3, double t4) {
+  return dvd(sub(add(sub(mul(48.0, t4), mul(p.w3[k], t3)), mul(p.w2[k], t2)), mul(p.w1[k], th)), p.den[k]);
+}
+
+// Eq. 17 for one velocity with component signs XS, YS (fq: its plane at the node), fe its f_eq, nuh line IV's factor.
+template <int XS, int YS>
+__device__ __forceinline__ double update_one(const double* __restrict__ fq, int pitch, const Params& p, int k,
+                                             double fe, const double (&nuh)[2]) {
+  constexpr int l = XS != 0 && YS != 0;
+  const double f0 = fq[0];
+  double acc = sub(f0, mul(p.r, sub(f0, fe)));
+#pragma unroll
+  for (int a = 0; a < 2; ++a) {
+    const int sg = a == 0 ? XS : YS, st = a == 0 ? 1 : pitch;
+    const double c1 = sg == 0 ? 0.0 : p.c1[a][k][l], c2 = sg == 0 ? 0.0 : p.c2[a][k][l], c3 = sg == 0 ? 0.0 : p.c3[a][k][l];
+    const double fp1 = fq[st], fm1 = fq[-st], fp2 = fq[2 * st], fm2 = fq[-2 * st];
+    const double cu = add(sub(fp1, mul(2.0, f0)), fm1);
+    acc = sub(acc, mul(sg < 0 ? -c1 : c1, sub(fp1, fm1)));
+    if (!(p.flags & F_NO_LW)) acc = add(acc, mul(c2, cu));
+    if (!(p.flags & F_NO_DISP))
+      acc = add(acc, mul(sg < 0 ? -c3 : c3, sub(add(sub(fp2, mul(2.0, fp1)), mul(2.0, fm1)), fm2)));
+    if (!(p.flags & F_NO_VISC)) acc = add(acc, mul(nuh[a], cu));
+  }
+  return acc;
 }
 
 template <int QQ>
@@ -217,10 +271,10 @@ __global__ void k_moments(const double* __restrict__ f, Grid g, unsigned* __rest
   mplane(g, 3)[off] = m.T;
 }
 
-// Pass 2: Eq. 17 at every interior node.
+// Pass 2: Eq. 17 at every interior node, a warp for 32 nodes of a row and one ring (threadIdx.y).
 __global__ void __launch_bounds__(128) k_update(const double* __restrict__ f, double* __restrict__ fn, Grid g,
                                                 Params p, unsigned* __restrict__ health) {
-  const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y * blockDim.y + threadIdx.y;
+  const int gx = blockIdx.x * 32 + threadIdx.x, gy = blockIdx.y + blockIdx.z * gridDim.y, K = threadIdx.y;
   if (gx >= g.nx || gy >= g.ny) return;
   const long long off = (long long)(gy + NG) * g.pitch + (gx + NG);
   const double* Mn = mplane(g, 0);
@@ -230,9 +284,7 @@ __global__ void __launch_bounds__(128) k_update(const double* __restrict__ f, do
   m.ux = mplane(g, 1)[off];
   m.uy = mplane(g, 2)[off];
   m.T = MT[off];
-  double F[5];
-  weights(m.T, F);
-  double sw[2], kap[2];
+  double nuh[2];
   unsigned bits = 0;
 #pragma unroll
   for (int a = 0; a < 2; ++a) {
@@ -240,15 +292,48 @@ __global__ void __launch_bounds__(128) k_update(const double* __restrict__ f, do
     const double Pp = mul(Mn[off + st], MT[off + st]);
     const double P0 = mul(m.n, m.T);
     const double Pm = mul(Mn[off - st], MT[off - st]);
-    sw[a] = (p.flags & F_SWITCH_CONST)
-                ? p.lam
-                : mul(p.lam, fabs(dvd(add(sub(Pp, mul(2.0, P0)), Pm), add(add(Pp, mul(2.0, P0)), Pm))));
-    kap[a] = dvd(mul(a == 0 ? m.ux : m.uy, p.dt), p.dr[a]);
-    if (fabs(kap[a]) > 1.0) bits |= H_KAPPA;
+    const double sw = (p.flags & F_SWITCH_CONST)
+                          ? p.lam
+                          : mul(p.lam, fabs(dvd(add(sub(Pp, mul(2.0, P0)), Pm), add(add(Pp, mul(2.0, P0)), Pm))));
+    const double ak = fabs(dvd(mul(a == 0 ? m.ux : m.uy, p.dt), p.dr[a]));
+    if (ak > 1.0) bits |= H_KAPPA;
+    nuh[a] = mul(mul(mul(sw, ak), sub(1.0, ak)), 0.5);
   }
-  const double r = dvd(p.dt, p.tau);
-  update_all<0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21, 22, 23, 24, 25, 26, 27, 28,
-             29, 30, 31, 32>(f, fn, g, p, off, gx, gy, ghost_own(g, gx, gy), m, F, r, sw, kap);
+  const GhostOwn go = ghost_own(g, gx, gy);
+  const EqNode e = eq_node(m.ux, m.uy, m.T);
+  const double t2 = mul(m.T, m.T), t3 = mul(t2, m.T), t4 = mul(t3, m.T);
+  double Fk;
+  if (K == 0) {  // and the rest velocity, whose weight needs all four
+    double sumF = 0.0;
+    Fk = weight(p, 0, m.T, t2, t3, t4);
+    sumF = add(sumF, Fk);
+#pragma unroll 1
+    for (int k = 1; k < 4; ++k) sumF = add(sumF, weight(p, k, m.T, t2, t3, t4));
+    double b0, unused;
+    brackets(e, add(mul(0.0, m.ux), mul(0.0, m.uy)), b0, unused);
+    const double fe = mul(mul(m.n, sub(1.0, mul(8.0, sumF))), b0);
+    store_node<double, 0>(fn, g, gx, gy, go, update_one<0, 0>(f + off, g.pitch, p, 0, fe, nuh));
+  } else {
+    Fk = weight(p, K, m.T, t2, t3, t4);
+  }
+  const double nF = mul(m.n, Fk), v = speed(K), vd = mul(v, __dsqrt_rn(0.5));
+  const double* fr = f + (long long)(1 + 8 * K) * g.plane + off;
+  double out[8];
+  auto pair = [&](auto xs, auto ys, int dp, int dm, double vu) {
+    constexpr int X = decltype(xs)::value, Y = decltype(ys)::value;
+    double bp, bm;
+    brackets(e, vu, bp, bm);
+    out[dp] = update_one<X, Y>(fr + dp * g.plane, g.pitch, p, K, mul(nF, bp), nuh);
+    out[dm] = update_one<-X, -Y>(fr + dm * g.plane, g.pitch, p, K, mul(nF, bm), nuh);
+  };
+  using P = std::integral_constant<int, 1>;
+  using Z = std::integral_constant<int, 0>;
+  using M = std::integral_constant<int, -1>;
+  pair(P{}, Z{}, 7, 3, add(mul(v, m.ux), mul(0.0, m.uy)));
+  pair(P{}, P{}, 0, 4, add(mul(vd, m.ux), mul(vd, m.uy)));
+  pair(Z{}, P{}, 1, 5, add(mul(0.0, m.ux), mul(v, m.uy)));
+  pair(M{}, P{}, 2, 6, add(mul(-vd, m.ux), mul(vd, m.uy)));
+  store_ring<double>(fn, g, gx, gy, go, K, out);
   if (bits) atomicOr(health, bits);
 }
 
@@ -316,21 +401,46 @@ __global__ void k_macro(const double* __restrict__ f, Grid g, double* __restrict
 }  // namespace strict
 }  // namespace
 
-cudaError_t launch_step_strict(const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
-                               cudaStream_t s) {
-  if (!g.mom) return cudaErrorInvalidValue;
+// Params with the header's operations, each rounded by itself on every host (no contraction).
+static strict::Params strict_params(const Grid& g, const Coeffs& c) {
+  auto mul = [](double a, double b) { volatile double r = a * b; return (double)r; };
+  auto add = [](double a, double b) { volatile double r = a + b; return (double)r; };
+  auto sub = [](double a, double b) { volatile double r = a - b; return (double)r; };
   strict::Params p;
   p.dt = c.sdt;
-  p.tau = c.stau;
   p.dr[0] = c.sdr[0];
   p.dr[1] = c.sdr[1];
   p.lam = c.lam;
+  p.r = c.sdt / c.stau;
   p.flags = g.flags;
+  const double s = std::sqrt(0.5);
+  for (int k = 0; k < 4; ++k) {
+    const double v = speed(k), va = speed((k + 1) % 4), vb = speed((k + 2) % 4), vc = speed((k + 3) % 4);
+    const double v2 = mul(v, v), a = mul(va, va), b = mul(vb, vb), d = mul(vc, vc);
+    p.den[k] = mul(mul(mul(v2, sub(v2, a)), sub(v2, b)), sub(v2, d));
+    p.w3[k] = mul(6.0, add(add(a, b), d));
+    p.w2[k] = add(add(mul(a, b), mul(b, d)), mul(d, a));
+    p.w1[k] = mul(mul(a, b), d) / 4.0;
+    for (int ax = 0; ax < 2; ++ax)
+      for (int l = 0; l < 2; ++l) {
+        const double cc = mul(l == 0 ? v : mul(v, s), c.sdt) / p.dr[ax];
+        p.c1[ax][k][l] = cc / 2.0;
+        p.c2[ax][k][l] = mul(cc, cc) / 2.0;
+        p.c3[ax][k][l] = mul(cc, sub(1.0, mul(cc, cc))) / 12.0;
+      }
+  }
+  return p;
+}
+
+cudaError_t launch_step_strict(const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
+                               cudaStream_t s) {
+  if (!g.mom) return cudaErrorInvalidValue;
+  const strict::Params p = strict_params(g, c);
   dim3 mb(32, 4), mg((g.nx + 2 + 31) / 32, (g.ny + 2 + 3) / 4);
   strict::k_moments<<<mg, mb, 0, s>>>(static_cast<const double*>(f), g, health);
-  dim3 ub(32, 4);
-  strict::k_update<<<grid2d(g, ub), ub, 0, s>>>(static_cast<const double*>(f), static_cast<double*>(fn), g, p,
-                                                health);
+  const unsigned rows = (unsigned)g.ny < 65535u ? (unsigned)g.ny : 65535u;
+  const dim3 ug((unsigned)((g.nx + 31) / 32), rows, ((unsigned)g.ny + rows - 1u) / rows);
+  strict::k_update<<<ug, dim3(32, 4), 0, s>>>(static_cast<const double*>(f), static_cast<double*>(fn), g, p, health);
   return cudaGetLastError();
 }
 
