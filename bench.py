@@ -14,9 +14,10 @@ above the 129 MB L2, so no L2 flush is needed between steps.
   resident in HBM.
 - e2e: the public call sequence with pinned host buffers inside the timed region:
   fdlbm_set_macro (H2D), fdlbm_step(K), fdlbm_get_macro (D2H).
-- roofline: the fused step kernel against the FP64 pipe (2 FP64 instructions per clock per SM,
-  the nominal 1.25 TFLOP/s). FP64 on this part issues ~60x slower than FP32, so the kernel is
-  bound by FP64 issue, not HBM. The HBM figures are reported beside it.
+- roofline: the fused step kernel against instruction issue (4 warp instructions per clock per SM)
+  where its instruction count is known, else against the FP64 pipe (2 FP64 instructions per clock
+  per SM, the nominal 1.25 TFLOP/s). No kernel here is bound by HBM; the FP64-pipe and HBM figures
+  are reported beside it.
 - cpu_baseline: the FP64 CPU oracle, timed on a bounded sample of the same workload.
 
 N > 1 (torchrun): every rank runs an independent replica with its own seed (weak scaling, no
@@ -41,42 +42,41 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# FP64 arithmetic instructions (DADD + DFMA + DMUL) per site update, each node's moments counted
-# once: ncu thread-level counts of the split step's two kernels, whose sum is the fused step's
-# work without the moments of the tile ring (see profiles/). FP32 storage sums its moments in
-# 64-bit fixed point on the integer pipes, hence the lower count (FP32 storage: 130 update +
-# 15 moments; FP64: 481 + 89). FNEQ32: ncu's count of k_step_fneq per site (the equilibrium rebuilt
-# on each tile's halo before the stencil and formed again from the new moments). fp32dw (the
-# double-word equilibrium): 15 for the moments and 4 to split the macros into double words (ncu:
+# FP64 arithmetic instructions per site update (ncu, sm__inst_executed_pipe_fp64 x 32 over the sites): fp32
+# (k_step_tma) and fp64 (k_step_fx) form moments and f_eq (fp64: Eq. 17 too) in fixed point on the integer
+# pipes; 66 and 96 counted, of which 6 and 4 for the tile ring's moments. FNEQ32: ncu's count of k_step_fneq per
+# site (the equilibrium rebuilt on each tile's halo before the stencil and formed again from the new moments).
+# fp32dw (the double-word equilibrium): 15 for the moments and 4 to split the macros into double words (ncu:
 # 23.9 with the tile ring's moments).
-FP64_OPS_PER_LUP = {"fp64": 570, "fp32": 145, "fneq32": 927, "fp32dw": 19}
+FP64_OPS_PER_LUP = {"fp64": 92, "fp32": 60, "fneq32": 927, "fp32dw": 19}
 # DRAM bytes (read + write) per site update of one step's launches (k_step, or k_moments +
 # k_update), by (precision, tile variant): ncu dram__bytes_read.sum + dram__bytes_write.sum of one
 # step of this bench's 4096^2 workload (single-pass capture), divided by the sites. Reported as roofline.traffic when the autotuner
 # picks the captured variant, else null.
-TRAFFIC_B_PER_SITE = {("fp32", 2): 268.5, ("fp32", 6): 267.6, ("fp32", 11): 467.8, ("fp64", 7): 836.7,
-                      ("fp64", 10): 873.5, ("fp32dw", 6): 266.3, ("fp32dw", 12): 263.1}
-# Warp instructions issued per site update (ncu smsp__inst_executed over the sites, 2048^2, same
-# kernels), by (precision, tile variant): the double-word step binds on instruction issue, whose
-# peak is 4 warp instructions per clock per SM (one per scheduler).
-WARP_INST_PER_SITE = {("fp32", 6): 121.6, ("fp32dw", 6): 131.3, ("fp32dw", 12): 125.0}
+TRAFFIC_B_PER_SITE = {("fp32", 2): 268.5, ("fp32", 6): 267.6, ("fp32", 11): 467.8, ("fp32", 12): 263.1,
+                      ("fp32dw", 6): 266.3, ("fp32dw", 12): 263.1}
+# Warp instructions issued per site update (ncu smsp__inst_executed over the sites, 2048^2; fp64 1024^2), by
+# (precision, tile variant): these steps bind on instruction issue, whose peak is 4 warp instructions per
+# clock per SM (one per scheduler). FP64 storage serves variants 2, 4-7, 10 and 11 with one kernel.
+WARP_INST_PER_SITE = {("fp32", 12): 138.0, ("fp32dw", 6): 131.3, ("fp32dw", 12): 125.0}
+WARP_INST_PER_SITE.update({("fp64", v): 324.3 for v in (2, 4, 5, 6, 7, 10, 11)})
 ISSUE_PER_CLK_SM = 4.0
-DTYPE = {"fp64": "f64", "fp32": "f32-store/fixed-point+f64-moments/f64-feq",
+DTYPE = {"fp64": "f64", "fp32": "f32-store/fixed-point+f64-moments/fixed-point-feq",
          "fneq32": "f64-macros+f32-fneq/f64-step", "fp32dw": "f32-store/df32-feq"}
-# Variants that split a step into two launches (moment pass + update pass). Their minimum bytes per
+# Variants that split a step into two launches (moment pass + update pass; FP64 storage runs its fused step). Their minimum bytes per
 # site update: f read twice and written once, the moment buffer (4 FP64 + P) written and read.
 SPLIT_VARIANTS = (10, 11)
 # Variants that run all the steps of a call in one cooperative launch (up to 4096 steps each).
 PERSISTENT_VARIANTS = (13, 14)
 GRAPH_VARIANT = 15  # the ring-parallel step launched from captured CUDA graphs
-BYTES_PER_LUP_SPLIT = {"fp64": 3 * 33 * 8 + 2 * (4 * 8 + 8), "fp32": 3 * 33 * 4 + 2 * (4 * 8 + 4),
+BYTES_PER_LUP_SPLIT = {"fp32": 3 * 33 * 4 + 2 * (4 * 8 + 4),
                        "fp32dw": 3 * 33 * 4 + 2 * (4 * 8 + 4)}
 # Minimum HBM bytes per site update: read and write all 33 f once.
 BYTES_PER_LUP = {"fp64": 2 * 33 * 8, "fp32": 2 * 33 * 4, "fneq32": 2 * (33 * 4 + 4 * 8), "fp32dw": 2 * 33 * 4}
 # FP64 instructions (DADD + DFMA + DMUL) per amplification-matrix spectrum of the von Neumann
 # tool on the Sec. 4 sweep: ncu thread-level counts of k_vn divided by the cases. They include the
 # rotation parameters every lane computes alike, so they bound the algorithmic work from above.
-FP64_OPS_PER_VN_MATRIX = 15.48e6
+FP64_OPS_PER_VN_MATRIX = 11.04e6
 # FP64 issue peak: 2 instructions per clock per SM, i.e. the nominal 1.25 TFLOP/s at 2.07 GHz
 # (ncu's pct-of-peak for the FP64 pipe agrees with it).
 FP64_OPS_PER_CLK_SM = 2.0
@@ -631,10 +631,17 @@ def main():
     fp64_measured = F.fdlbm_fp64_rate(20000, stream) / 1e9
     site_rate = w.nx * w.ny / (per_launch_ms * 1e-3)
     achieved = FP64_OPS_PER_LUP[prec_name] * site_rate / 1e9
-    split = variant in SPLIT_VARIANTS
+    split = variant in SPLIT_VARIANTS and prec_name != "fp64"
     hbm_gbs = (BYTES_PER_LUP_SPLIT if split else BYTES_PER_LUP)[prec_name] * site_rate / 1e9
     tb = TRAFFIC_B_PER_SITE.get((prec_name, variant)) if (w.nx, w.ny) == (4096, 4096) else None
     traffic = tb * w.nx * w.ny if tb else None
+    issue = issue_roofline(prec_name, variant, site_rate, sm_mhz)
+    fp64_pipe = {
+        "achieved": achieved, "peak": fp64_peak, "unit": "G FP64-pipe ops/s", "frac": achieved / fp64_peak,
+        "peak_derivation": "2 FP64 ops/clk/SM (nominal 1.25 TFLOP/s) x 152 SMs x %.0f MHz sampled" % sm_mhz,
+        "peak_measured": fp64_measured, "frac_of_measured": achieved / fp64_measured,
+        "peak_measured_how": "fdlbm_fp64_rate: 8 independent FMA chains per thread, 8 CTAs x 256 "
+                             "threads per SM, CUDA events, right after the timed steps"}
 
     line = {
         "metric": "GLUPS", "value": glups, "unit": "GLUPS", "n_gpus": world, "steps": args.steps,
@@ -650,20 +657,17 @@ def main():
         "roofline": {"bound": "alu", "kernel": "k_step_fneq (FNEQ32 step)" if prec_name == "fneq32" else
                      "k_moments + k_update (split step)" if split else
                      "k_step_tma (fused step, tile by tensor copy)" if variant == 12 and prec_name in ("fp32", "fp32dw")
-                     else "k_persist_rp / k_persist_tile (persistent steps)" if variant in PERSISTENT_VARIANTS
+                     else "k_persist_* (persistent steps)" if variant in PERSISTENT_VARIANTS
                      and prec_name in ("fp32", "fp64")
-                     else "k_step_rp (ring-parallel steps replayed from CUDA graphs of 32)" if variant == GRAPH_VARIANT
-                     and prec_name in ("fp32", "fp64") else "k_step (fused step)",
-                     "achieved": achieved,
-                     "peak": fp64_peak, "unit": "G FP64-pipe ops/s", "frac": achieved / fp64_peak,
+                     else "small-grid steps replayed from CUDA graphs of 32" if variant == GRAPH_VARIANT
+                     and prec_name in ("fp32", "fp64") else "k_step_fx (fused step, fixed point)"
+                     if prec_name == "fp64" else "k_step (fused step)",
+                     **{k: (issue or fp64_pipe)[k] for k in ("achieved", "peak", "unit", "frac", "peak_derivation")},
                      "traffic": traffic, "traffic_unit": "bytes per step (ncu DRAM read + write of its launches)",
-                     "peak_derivation": "2 FP64 ops/clk/SM (nominal 1.25 TFLOP/s) x 152 SMs x %.0f MHz sampled" % sm_mhz,
-                     "peak_measured": fp64_measured, "frac_of_measured": achieved / fp64_measured,
-                     "peak_measured_how": "fdlbm_fp64_rate: 8 independent FMA chains per thread, 8 CTAs x 256 "
-                                          "threads per SM, CUDA events, right after the timed steps",
+                     "fp64_pipe": fp64_pipe,
                      "hbm": {"achieved_gbs": hbm_gbs, "peak_gbs": peaks.get("hbm_gbs"), "peak_kind": peak_kind,
                              "frac": hbm_gbs / peaks.get("hbm_gbs", 6800.0)},
-                     "issue": issue_roofline(prec_name, variant, site_rate, sm_mhz)},
+                     "issue": issue},
         "clocks": clocks,
         "e2e": {"value": e2e_glups, "unit": "GLUPS", "h2d_bytes_per_step": macro_bytes / args.steps,
                 "d2h_bytes_per_step": macro_bytes / args.steps, "status": int(rc),
