@@ -258,7 +258,7 @@ int default_variant(const fdlbm_config* c) {
     // Times per step on a GB300 (us). The 4 x 4 tile (V_RP8x4; two per SM, 4864 sites at a time) is the shortest
     // step: 400 x 4 9.7 against 13.9 with 8 x 4 tiles, 2000 x 4 18.4 against 22.6; in its third round, at 4000 x 4,
     // 32.9 against 23.6. The 8 x 4 tile holds 19456 sites at a time: 200 x 200 52.6 against 62.6 with 32 x 8 tiles,
-    // 16384 x 4 74.2 against 60.6 with 32 x 4. Beyond, 32 x 8 (2048^2 2170, 32 x 4 2540), a tube's 4 rows 32 x 4.
+    // 16384 x 4 74.2 against 53.0 with 32 x 4. Beyond, 32 x 8 (2048^2 2170, 32 x 4 2540), a tube's 4 rows 32 x 4.
     if (sites <= 9728) return V_RP8x4;
     if (sites <= kF64SmallSites) return V_RP16x4;
     return c->ny <= 4 ? V_T32x4 : V_T32x16;

@@ -435,14 +435,33 @@ struct FxBox {
   }
 };
 
+// The cells that a tile converts: its box, or (DUP), where it holds the whole height of a y-periodic grid, the grid's
+// rows with their halo columns, each stored again in the ghost row that copies it.
+template <int TW, int TH, bool DUP>
+struct FxCells {
+  using X = FxBox<TW, TH>;
+  static constexpr int N = DUP ? (TW + 4) * TH : X::CELLS, NV = (N + 31) / 32;
+  __device__ static int2 cell(int idx) {
+    if constexpr (DUP) return make_int2(idx % (TW + 4), idx / (TW + 4) + 2);
+    else return X::cell(idx);
+  }
+  __device__ static void put(int2* __restrict__ box, int2 p, int2 w) {
+    box[p.y * X::BW + p.x] = w;
+    if constexpr (DUP) {
+      if (p.y < 4) box[(p.y + TH) * X::BW + p.x] = w;
+      if (p.y >= TH) box[(p.y - TH) * X::BW + p.x] = w;
+    }
+  }
+};
+
 // One warp converts one plane into its box, from the lane's cells' values v (a cell that no stencil reads
 // takes another cell's value); returns the plane's class entry.
-template <int TW, int TH, bool COH>
+template <int TW, int TH, bool COH, bool DUP = false>
 __device__ __forceinline__ int convert_plane(const double* __restrict__ pl, const Grid& g, int x0, int y0, int lane,
-                                             const double (&v)[(FxBox<TW, TH>::CELLS + 31) / 32],
-                                             int2* __restrict__ box) {
+                                             const double (&v)[FxCells<TW, TH, DUP>::NV], int2* __restrict__ box) {
   using X = FxBox<TW, TH>;
-  constexpr int NV = (X::CELLS + 31) / 32;
+  using C = FxCells<TW, TH, DUP>;
+  constexpr int NV = C::NV;
   unsigned amax = 0u, amin = 0x7fffffffu;
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
@@ -456,39 +475,40 @@ __device__ __forceinline__ int convert_plane(const double* __restrict__ pl, cons
   if (cl == cm) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int2 p = X::cell(lane + 32 * i);
+      const int2 p = C::cell(lane + 32 * i);
       const unsigned a = (unsigned)__double2hiint(v[i]) & 0x7fffffffu;
       const L28 t = l28(val_fixed(v[i], (int)(a >> 20) - (4 * cl - 5)));
-      if (lane + 32 * i < X::CELLS) box[p.y * X::BW + p.x] = make_int2(t.h, t.l);
+      if (lane + 32 * i < C::N) C::put(box, p, make_int2(t.h, t.l));
     }
     return cl;
   }
   if constexpr (NV <= 4) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
-      const int2 p = X::cell(lane + 32 * i);
+      const int2 p = C::cell(lane + 32 * i);
       const int2 w = mixed_entry(v[i], cl);
-      if (lane + 32 * i < X::CELLS) box[p.y * X::BW + p.x] = w;
+      if (lane + 32 * i < C::N) C::put(box, p, w);
     }
   } else {  // the cells again, in a loop
 #pragma unroll 1
-    for (int i = lane; i < X::CELLS; i += 32) {
-      const int2 p = X::cell(i);
+    for (int i = lane; i < C::N; i += 32) {
+      const int2 p = C::cell(i);
       if (X::needed(g, x0 + p.x, y0 + p.y))
-        box[p.y * X::BW + p.x] = mixed_entry(ldf<COH>(pl + (long long)(y0 + p.y) * g.pitch + x0 + p.x), cl);
+        C::put(box, p, mixed_entry(ldf<COH>(pl + (long long)(y0 + p.y) * g.pitch + x0 + p.x), cl));
     }
   }
   return cl | kMixed;
 }
-template <int TW, int TH>
+template <int TW, int TH, bool DUP = false>
 __device__ __forceinline__ void plane_cells(const Grid& g, int x0, int y0, int lane,
-                                            int (&src)[(FxBox<TW, TH>::CELLS + 31) / 32]) {
+                                            int (&src)[FxCells<TW, TH, DUP>::NV]) {
   using X = FxBox<TW, TH>;
+  using C = FxCells<TW, TH, DUP>;
 #pragma unroll
-  for (int i = 0; i < (X::CELLS + 31) / 32; ++i) {
-    const int2 p = X::cell(lane + 32 * i);
+  for (int i = 0; i < C::NV; ++i) {
+    const int2 p = C::cell(lane + 32 * i);
     const int cx = x0 + p.x, cy = y0 + p.y;
-    const bool use = lane + 32 * i < X::CELLS && X::needed(g, cx, cy);
+    const bool use = lane + 32 * i < C::N && X::needed(g, cx, cy);
     src[i] = use ? cy * g.pitch + cx : (y0 + NG) * g.pitch + x0 + NG;
   }
 }
@@ -563,8 +583,8 @@ struct FxTile {
 
 // One tile of the FP64 step, one lane per node, the rings one after the other. A tile that holds a
 // y-periodic grid's whole height takes its two ghost rows' macros from the interior rows they copy.
-template <int TW, int TH, bool COH>
-__device__ __forceinline__ void fx_tile(const double* __restrict__ f, double* __restrict__ fn, const Grid& g,
+template <int TW, int TH, bool COH, bool DUP>
+__device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, double* __restrict__ fn, const Grid& g,
                                         const Coeffs& c, unsigned* __restrict__ health, int tile_x, int tile_y,
                                         FxTile<TW, TH>& sm) {
   using S = FxTile<TW, TH>;
@@ -634,18 +654,19 @@ __device__ __forceinline__ void fx_tile(const double* __restrict__ f, double* __
       nuyi = nu_fixed(dnuy, c.xS);
     }
   }
-  int src[(X::CELLS + 31) / 32];
-  plane_cells<TW, TH>(g, x0, y0, lane, src);
+  constexpr int NV = FxCells<TW, TH, DUP>::NV;
+  int src[NV];
+  plane_cells<TW, TH, DUP>(g, x0, y0, lane, src);
 #pragma unroll 1
   for (int K = 0; K < 4; ++K) {
     if (K) __syncthreads();  // the previous planes have been read
 #pragma unroll 1
     for (int q = warp; q < 8; q += NT / 32) {
       const double* pl = f + (long long)(1 + 8 * K + q) * g.plane;
-      double v[(X::CELLS + 31) / 32];
+      double v[NV];
 #pragma unroll
-      for (int i = 0; i < (X::CELLS + 31) / 32; ++i) v[i] = ldf<COH>(pl + src[i]);
-      const int cl = convert_plane<TW, TH, COH>(pl, g, x0, y0, lane, v, sm.box[q]);
+      for (int i = 0; i < NV; ++i) v[i] = ldf<COH>(pl + src[i]);
+      const int cl = convert_plane<TW, TH, COH, DUP>(pl, g, x0, y0, lane, v, sm.box[q]);
       if (lane == 0) sm.cls[q] = cl;
     }
     __syncthreads();
@@ -699,6 +720,19 @@ __device__ __forceinline__ void fx_tile(const double* __restrict__ f, double* __
   if (mine)
     rest_update<COH>(f, fn, g, c, off, gx, gy, go, fma(-8.0, snF, c.r * sm.n[so]) * e.A0d, dnux, dnuy);
   if (bits) atomicOr(health, bits);
+}
+
+// 4-row tubes are the tiles whose halo rows weigh most (272 converted cells for 128 nodes, 144 without): the 32 x 4
+// tile has a form of its own for them (16384 x 4: 60.6 -> 53.0 us per step; 40000 x 4: 124 -> 115).
+template <int TW, int TH, bool COH>
+__device__ __forceinline__ void fx_tile(const double* __restrict__ f, double* __restrict__ fn, const Grid& g,
+                                        const Coeffs& c, unsigned* __restrict__ health, int tile_x, int tile_y,
+                                        FxTile<TW, TH>& sm) {
+  if constexpr (TH == 4) {
+    if (g.ny == TH && g.bc[2] == BC_PERIODIC && g.bc[3] == BC_PERIODIC)
+      return fx_tile_body<TW, TH, COH, true>(f, fn, g, c, health, tile_x, tile_y, sm);
+  }
+  fx_tile_body<TW, TH, COH, false>(f, fn, g, c, health, tile_x, tile_y, sm);
 }
 
 // ---------------------------------------------------------------------------------------------
