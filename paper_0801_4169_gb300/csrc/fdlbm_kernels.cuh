@@ -359,12 +359,45 @@ __device__ __forceinline__ long long to_fix(float x, int emax) {
   const FixTerm t = fix_term<FULL>(x, emax);
   return (long long)t.sm * t.p;
 }
-// V * 2^e2, rounded to nearest even, built from the integer's bits (|V| < 2^63, normal result).
-__device__ __forceinline__ double fix_to_f64(long long V, int e2) { return fx::to_f64(V, e2); }
+// V * 2^e2, rounded to nearest even, built from the integer's bits (|V| < 2^63, normal result). ASM: see sum_mad.
+template <bool ASM>
+__device__ __forceinline__ double fix_to_f64(long long V, int e2) {
+  if constexpr (ASM) return fx::to_f64(V, e2);
+  if (V == 0) return 0.0;
+  const unsigned long long sgn = (unsigned long long)V & 0x8000000000000000ull;
+  const unsigned long long A = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
+  const int lz = __clzll((long long)A);  // >= 1
+  const unsigned long long U = A << (lz - 1);  // leading one at bit 62
+  // round to nearest even at bit 10: add 2^9 - 1 plus the lowest kept bit, then drop the 10 bits
+  // (no overflow: U < 2^63). M has its leading one at bit 52, or is 2^53 after a carry.
+  const unsigned long long M = (U + 0x1ffull + ((U >> 10) & 1ull)) >> 10;
+  const unsigned long long E = (unsigned long long)(1086 - lz + e2);  // biased exponent
+  // the leading one (bit 52) adds the last 1 to the exponent field; a carry to 2^53 adds one more,
+  // which is the correct result
+  return __longlong_as_double((long long)(sgn | (((E - 1ull) << 52) + M)));
+}
 struct RingFix {
   long long S, AX, DX, AY, DY;
 };
-template <bool FULL = true>
+// The sums' multiply-adds and conversions written out (ASM), or left to the compiler, which serves the double-word
+// kernels better: 16384 x 4 26.8 against 28.7 us (2048^2 by tensor copy 0.622 against 0.624 ms), where f_eq in fixed
+// point takes 0.911 against 0.838 ms at 2048^2. The same integers.
+template <bool ASM>
+__device__ __forceinline__ long long sum_mad(int a, int b, long long c) {
+  if constexpr (ASM) return fx::mad(a, b, c);
+  else return (long long)a * b + c;
+}
+template <bool ASM>
+__device__ __forceinline__ long long sum_mad_u(unsigned a, unsigned b, long long c) {
+  if constexpr (ASM) return fx::mad_u(a, b, c);
+  else return (long long)((unsigned long long)a * b + (unsigned long long)c);
+}
+template <bool ASM>
+__device__ __forceinline__ long long sum_mad_small(int a, long long v, long long c) {
+  if constexpr (ASM) return fx::mad_small((unsigned)a, v, c);
+  else return (long long)a * v + c;
+}
+template <bool FULL = true, bool ASM = true>
 __device__ __forceinline__ RingFix ring_fix(const float (&x)[8], int emax) {
   FixTerm t[8];
 #pragma unroll
@@ -372,11 +405,11 @@ __device__ __forceinline__ RingFix ring_fix(const float (&x)[8], int emax) {
   RingFix r;
   r.S = 0;
 #pragma unroll
-  for (int d = 0; d < 8; ++d) r.S = fx::mad(t[d].sm, t[d].p, r.S);
-  r.AX = fx::mad(t[3].sm, -t[3].p, fx::mad(t[7].sm, t[7].p, 0));
-  r.AY = fx::mad(t[5].sm, -t[5].p, fx::mad(t[1].sm, t[1].p, 0));
-  const long long a = fx::mad(t[4].sm, -t[4].p, fx::mad(t[0].sm, t[0].p, 0));
-  const long long b = fx::mad(t[2].sm, -t[2].p, fx::mad(t[6].sm, t[6].p, 0));
+  for (int d = 0; d < 8; ++d) r.S = sum_mad<ASM>(t[d].sm, t[d].p, r.S);
+  r.AX = sum_mad<ASM>(t[3].sm, -t[3].p, sum_mad<ASM>(t[7].sm, t[7].p, 0));
+  r.AY = sum_mad<ASM>(t[5].sm, -t[5].p, sum_mad<ASM>(t[1].sm, t[1].p, 0));
+  const long long a = sum_mad<ASM>(t[4].sm, -t[4].p, sum_mad<ASM>(t[0].sm, t[0].p, 0));
+  const long long b = sum_mad<ASM>(t[2].sm, -t[2].p, sum_mad<ASM>(t[6].sm, t[6].p, 0));
   r.DX = a + b;
   r.DY = a - b;
   return r;
@@ -389,24 +422,26 @@ __device__ __forceinline__ Mom nan_moments() {
 // The energy sum 10^4 sum_k v_k^2 S_k = sum_k V_k^2 S_k needs up to 71 bits, so each S_k is split
 // as hi 2^32 + lo (lo unsigned): EH = sum_k V_k^2 hi_k (|EH| < 2^41) and EL = sum_k V_k^2 lo_k
 // (< 2^52) are exact integers.
+template <bool ASM = true>
 __device__ __forceinline__ void energy_parts(int k, long long S, long long& EH, long long& EL) {
   const int v2 = speed_c(k) * speed_c(k);
-  EH = fx::mad((int)(S >> 32), v2, EH);
-  EL = fx::mad_u((unsigned)S, (unsigned)v2, EL);
+  EH = sum_mad<ASM>((int)(S >> 32), v2, EH);
+  EL = sum_mad_u<ASM>((unsigned)S, (unsigned)v2, EL);
 }
 // n, 100 jx, 100 jy and 10^4 sum |v|^2 f from the exact sums. EH 2^32 and EL convert to FP64
 // exactly (both below 2^53), so their one FP64 sum is the correctly rounded energy sum.
+template <bool ASM = true>
 __device__ __forceinline__ Mom fix_moments(long long N, long long Ax, long long Dx, long long Ay, long long Dy,
                                            long long EH, long long EL, int e2) {
   Mom m;
-  m.n = fix_to_f64(N, e2);
-  m.jx = fma(kS, fix_to_f64(Dx, e2), fix_to_f64(Ax, e2));
-  m.jy = fma(kS, fix_to_f64(Dy, e2), fix_to_f64(Ay, e2));
-  m.e2 = fix_to_f64(EH, e2 + 32) + fix_to_f64(EL, e2);
+  m.n = fix_to_f64<ASM>(N, e2);
+  m.jx = fma(kS, fix_to_f64<ASM>(Dx, e2), fix_to_f64<ASM>(Ax, e2));
+  m.jy = fma(kS, fix_to_f64<ASM>(Dy, e2), fix_to_f64<ASM>(Ay, e2));
+  m.e2 = fix_to_f64<ASM>(EH, e2 + 32) + fix_to_f64<ASM>(EL, e2);
   return m;
 }
 
-template <bool FULL>
+template <bool FULL, bool ASM>
 __device__ __forceinline__ Mom fix_node_moments(const float (&x)[Q], int emax) {
   const int e2 = emax - FIX_E2;
   long long N = to_fix<FULL>(x[0], emax), Ax = 0, Dx = 0, Ay = 0, Dy = 0, EH = 0, EL = 0;
@@ -415,21 +450,21 @@ __device__ __forceinline__ Mom fix_node_moments(const float (&x)[Q], int emax) {
     float g[8];
 #pragma unroll
     for (int d = 0; d < 8; ++d) g[d] = x[1 + 8 * k + d];
-    const RingFix r = ring_fix<FULL>(g, emax);
+    const RingFix r = ring_fix<FULL, ASM>(g, emax);
     N += r.S;
-    Ax = fx::mad_small(speed_c(k), r.AX, Ax);
-    Dx = fx::mad_small(speed_c(k), r.DX, Dx);
-    Ay = fx::mad_small(speed_c(k), r.AY, Ay);
-    Dy = fx::mad_small(speed_c(k), r.DY, Dy);
-    energy_parts(k, r.S, EH, EL);
+    Ax = sum_mad_small<ASM>(speed_c(k), r.AX, Ax);
+    Dx = sum_mad_small<ASM>(speed_c(k), r.DX, Dx);
+    Ay = sum_mad_small<ASM>(speed_c(k), r.AY, Ay);
+    Dy = sum_mad_small<ASM>(speed_c(k), r.DY, Dy);
+    energy_parts<ASM>(k, r.S, EH, EL);
   }
-  return fix_moments(N, Ax, Dx, Ay, Dy, EH, EL, e2);
+  return fix_moments<ASM>(N, Ax, Dx, Ay, Dy, EH, EL, e2);
 }
 
 // Moments of an FP32-storage node; jx, jy in hundredths and the energy in 10^-4 (to_macro<100>).
 // When the node's values are all normal and lie within 2^FIX_TOP of its largest (the usual case),
 // the terms take the short form; the results are the same.
-template <bool COH = false>
+template <bool COH = false, bool ASM = true>
 __device__ __forceinline__ Mom node_moments(const float* __restrict__ f, long long plane, long long off,
                                             const Coeffs& c) {
   float x[Q];
@@ -442,8 +477,8 @@ __device__ __forceinline__ Mom node_moments(const float* __restrict__ f, long lo
     emin = min(emin, e);
   }
   if (emax == 255) return nan_moments();
-  if (emin > 0 && emax - emin <= FIX_TOP) return fix_node_moments<false>(x, emax);
-  return fix_node_moments<true>(x, emax);
+  if (emin > 0 && emax - emin <= FIX_TOP) return fix_node_moments<false, ASM>(x, emax);
+  return fix_node_moments<true, ASM>(x, emax);
 }
 
 // (n, ux, uy, T, P) from the sums; T = (sum |v|^2 f)/(2n) - |u|^2/2  (Eq. 5 with P = nT). JS is
@@ -466,15 +501,15 @@ __device__ __forceinline__ Macro to_macro(const Mom& m) {
   o.P = m.n * o.T;
   return o;
 }
-template <bool COH = false>
+template <bool COH = false, bool ASM = true>
 __device__ __forceinline__ Macro node_macro(const double* __restrict__ f, long long plane, long long off,
                                             const Coeffs& c) {
   return to_macro<1>(node_moments<COH>(f, plane, off, c));
 }
-template <bool COH = false>
+template <bool COH = false, bool ASM = true>
 __device__ __forceinline__ Macro node_macro(const float* __restrict__ f, long long plane, long long off,
                                             const Coeffs& c) {
-  return to_macro<100>(node_moments<COH>(f, plane, off, c));
+  return to_macro<100>(node_moments<COH, ASM>(f, plane, off, c));
 }
 
 // Ring-parallel kernel: the macros of the quad's node, bit for bit those of node_macro. Each lane forms its
@@ -1095,7 +1130,7 @@ __device__ __forceinline__ void stage_feq(S* __restrict__ s_fe, int node, double
 // (local (1, 1)), stored if an update needs them: every interior node and the ghost layer next to
 // an edge, never a grid corner. Its loads take an address clamped into the padded grid, so that a
 // caller can run it branch-free on slots it does not need.
-template <typename S, int SW, bool COH>
+template <typename S, int SW, bool COH, bool ASM>
 __device__ __forceinline__ void moment_slot(const S* __restrict__ f, const Grid& g, const Coeffs& c, int x0, int y0,
                                             int lx, int ly, double (*s_n)[SW], double (*s_ux)[SW],
                                             double (*s_uy)[SW], double (*s_T)[SW], S (*s_P)[SW], unsigned& bits) {
@@ -1104,7 +1139,7 @@ __device__ __forceinline__ void moment_slot(const S* __restrict__ f, const Grid&
   const bool need = (inx && iny) || (iny && (gx == -1 || gx == g.nx)) || (inx && (gy == -1 || gy == g.ny));
   const int cx = min(max(gx, -1), g.nx), cy = min(max(gy, -1), g.ny);  // inside the padded grid
   const long long off = (long long)(cy + NG) * g.pitch + (cx + NG);
-  const Macro m = node_macro<COH>(f, g.plane, off, c);
+  const Macro m = node_macro<COH, ASM>(f, g.plane, off, c);
   if (need) {
     if (!macro_ok(m)) bits |= H_NUMERIC;
     s_n[ly][lx] = m.n;
@@ -1229,7 +1264,7 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
     const int idx = tid + k * NT;
     // the slots before the last always lie in the tile ring (no branch); the last one is guarded
     if (WRAPY ? idx >= nslot : ((k + 1) * NT > SW * SH && idx >= SW * SH)) continue;
-    moment_slot<S, SW, COH>(f, g, c, x0, y0, idx % SW, idx / SW + (wrap ? 1 : 0), s_n, s_ux, s_uy, s_T, s_P, bits);
+    moment_slot<S, SW, COH, !DW>(f, g, c, x0, y0, idx % SW, idx / SW + (wrap ? 1 : 0), s_n, s_ux, s_uy, s_T, s_P, bits);
   }
   if (wrap) {  // CTA-uniform
     __syncthreads();
@@ -1275,6 +1310,9 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
       snuy = (S)0.5 * thy * aky * ((S)1 - aky);
     }
     const S w0base = ((S)1 - SC::r(c)) - (S)2 * (snux + snuy);
+    typename std::conditional<DW, EqSiteDW, FeqNode>::type e;
+    if constexpr (DW) e = eq_site_dw(n, ux, uy, T, c);
+    else e = feq_node<S>(n, ux, uy, T, c);
     const long long off = (long long)(gy + NG) * g.pitch + (gx + NG);
     const GhostOwn go = ghost_own(g, gx, gy);
     // rest velocity: f_eq = n F_0 A0; c = 0 on both axes (line IV only)
@@ -1286,12 +1324,12 @@ __device__ __forceinline__ void step_tile(const S* __restrict__ f, S* __restrict
       store_node<S, 0>(fn, g, gx, gy, go, acc);
     };
     if constexpr (DW) {
-      const EqSiteDW e = eq_site_dw(n, ux, uy, T, c);
       rest(e.rest);
-#pragma unroll
-      for (int K = 0; K < 4; ++K) update_ring<S, COH>(K, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, COH>(0, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, COH>(1, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, COH>(2, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
+      update_ring<S, COH>(3, f, fn, g, c, off, gx, gy, go, e, w0base, snux, snuy);
     } else {
-      const FeqNode e = feq_node<S>(n, ux, uy, T, c);
       double snF = 0.0;
 #pragma unroll 1
       for (int K = 0; K < 4; ++K) {

@@ -72,6 +72,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int lim
 }
 
 // Moments of the node whose box entry (plane 0) is at s[idx]; same arithmetic as node_moments.
+template <bool ASM>
 __device__ __forceinline__ Macro box_macro(const float* __restrict__ s, int idx) {
   float x[Q];
   int emax = 1, emin = 255;
@@ -84,8 +85,8 @@ __device__ __forceinline__ Macro box_macro(const float* __restrict__ s, int idx)
   }
   Mom m;
   if (emax == 255) m = nan_moments();
-  else if (emin > 0 && emax - emin <= FIX_TOP) m = fix_node_moments<false>(x, emax);
-  else m = fix_node_moments<true>(x, emax);
+  else if (emin > 0 && emax - emin <= FIX_TOP) m = fix_node_moments<false, ASM>(x, emax);
+  else m = fix_node_moments<true, ASM>(x, emax);
   return to_macro<100>(m);
 }
 
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(kTW * kTH, MINB)
     const int gx = x0 + lx - 1, gy = y0 + ly - 1;
     const bool inx = gx >= 0 && gx < g.nx, iny = gy >= 0 && gy < g.ny;
     const bool need = (inx && iny) || (iny && (gx == -1 || gx == g.nx)) || (inx && (gy == -1 || gy == g.ny));
-    const Macro m = box_macro(s_f, (ly + 1) * kBW + (lx + 1));
+    const Macro m = box_macro<!DW>(s_f, (ly + 1) * kBW + (lx + 1));
     if (need) {
       if (!macro_ok(m)) bits |= H_NUMERIC;
       s_n[ly][lx] = m.n;
