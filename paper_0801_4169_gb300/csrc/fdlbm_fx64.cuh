@@ -142,7 +142,15 @@ __device__ __forceinline__ Macro macro_from_sums(const NodeSums& s, int ex) {
 template <bool COH>
 __device__ __noinline__ Macro node_macro_f64(const double* __restrict__ f, long long plane, long long off,
                                              const Coeffs& c) {
-  return to_macro<1>(node_moments<COH>(f, plane, off, c));
+  double S[4], X[4], Y[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    double x[8];
+#pragma unroll
+    for (int d = 0; d < 8; ++d) x[d] = ldf<COH>(f + (long long)(1 + 8 * k + d) * plane + off);
+    ring_sums(x, S[k], X[k], Y[k]);
+  }
+  return to_macro<1>(combine_rings(ldf<COH>(f + off), S, X, Y, c));
 }
 __device__ __forceinline__ bool mom_range(int emax) { return emax >= kMomEmin && emax < 2047 - 8; }
 template <bool COH>
