@@ -250,11 +250,11 @@ FX_HD Base base_of(double A0, double A1, double p0, double p1, double p2, double
   if (bits_of(A0) >> 63) b.A0f = -b.A0f;
   return b;
 }
-// a weight nF_k that the fixed-point form can take: 2^-60 < |nF_k| < 2^40
-FX_HD bool weight_ok(double nF) {
-  const unsigned f = abs_hi(nF);
-  return f > (1023u - 60u) << 20 && f < (1023u + 40u) << 20;
-}
+// A weight nF_k that the fixed-point form can take, for FP64 results: 2^-700 < |nF_k| < 2^700. Its exponent is part of
+// the results' scale alone, an integer; the limits keep the results normal.
+FX_HD bool weight_ok(double nF) { return abs_hi(nF) - ((1023u - 700u) << 20) < 1400u << 20; }
+// ... for FP32 results, whose scale is an FP32 number: 2^-60 < |nF_k| < 2^40
+FX_HD bool weight_ok_f32(double nF) { return abs_hi(nF) - ((1023u - 60u) << 20) < 100u << 20; }
 // es of ring k
 FX_HD int scale_of(const Base& b, int k) {
   const float v = k == 0 ? 1.0f : k == 1 ? 1.92f : k == 2 ? 2.99f : 4.49f;

@@ -702,15 +702,20 @@ __device__ __forceinline__ FeqNode feq_node(double n, double ux, double uy, doub
 // r n F_k (Eqs. 11-13) from r n theta. Where f_eq's brackets and the moments take the speeds as exact
 // decimals (FP64 storage), F_k's coefficients have to be theirs too: rounded to FP64 they violate the moment
 // identities by 2^-53 of f, always with the same sign. The rounded parts' polynomial, in FP32, enters with
-// the last operation.
+// the last operation: times r n theta's significand, whose exponent is put back on the product's bits, so that
+// densities outside FP32's range (number densities, a tenuous gas) get the same correction.
 template <bool EXACT>
 __device__ __forceinline__ double weight_poly(double rnth, double th, int K, const Coeffs& c) {
   const double P = fma(th, fma(th, fma(th, c.Fh[K][3], c.Fh[K][2]), c.Fh[K][1]), c.Fh[K][0]);
   if constexpr (!EXACT) return rnth * P;
   const float t = f64_trunc32(th), l = fmaf(t, fmaf(t, fmaf(t, c.Fl[K][3], c.Fl[K][2]), c.Fl[K][1]), c.Fl[K][0]);
-  const float corr = f64_trunc32(rnth) * l;
-  const double d = fabsf(corr) >= 1.17549435e-38f ? f32_to_f64_bits(corr) : 0.0;
-  return fma(rnth, P, d);
+  const unsigned hi = (unsigned)__double2hiint(rnth), lo = (unsigned)__double2loint(rnth);
+  const unsigned E = hi >> 20 & 0x7ffu;
+  const float corr = __uint_as_float((hi & 0x80000000u) | 0x3f800000u | (hi & 0xfffffu) << 3 | lo >> 29) * l;
+  const double d = f32_to_f64_bits(corr);
+  const double s = __hiloint2double(__double2hiint(d) + (int)((E - 1023u) << 20), __double2loint(d));
+  // the result stays normal: |corr| > 2^-126
+  return fma(rnth, P, fabsf(corr) >= 1.17549435e-38f && E - 150u < 1700u ? s : 0.0);
 }
 template <bool EXACT>
 __device__ __forceinline__ double ring_weight(const FeqNode& e, int K, const Coeffs& c) {
@@ -722,7 +727,7 @@ __device__ constexpr int dir_minus(int t) { return t == 0 ? 3 : t + 3; }
 // r f_eq of ring K's 8 directions; nF = ring_weight<false>(e, K, c). n..T: the node's macros (rare form).
 __device__ __forceinline__ void feq_ring(const FeqNode& e, int K, double nF, const Coeffs& c, double n, double ux,
                                          double uy, double T, float (&fe)[8]) {
-  if (__builtin_expect(e.b.ok && fx::weight_ok(nF), 1)) {
+  if (__builtin_expect(e.b.ok && fx::weight_ok_f32(nF), 1)) {
     const fx::RingFx r = fx::ring_shared(e.A0, e.es, nF, c.fxc[0][K]);
     const float up = fx::pow2_f32(r.ex + 36), down = fx::pow2_f32(r.ex + 4);
 #pragma unroll

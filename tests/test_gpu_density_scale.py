@@ -1,0 +1,44 @@
+"""The step is linear in f, so with f times a power of 16 every result is the same number times that power, bit for
+bit, as long as a node is computed in one and the same arithmetic at both scales. A state whose density leaves the
+range that the fixed-point form takes is computed in the FP64 form instead, seven times slower, and its rounding differs.
+Number densities (1e25 and more) and a tenuous gas are ordinary input."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from paper_0801_4169_gb300 import fdlbm as F  # noqa: E402
+
+PER, OUT, WALL = F.FDLBM_BC_PERIODIC, F.FDLBM_BC_OUTFLOW, F.FDLBM_BC_WALL
+
+
+def _state(nx, ny, seed):
+    """Smooth waves with a jump of density and pressure in the middle."""
+    rng = np.random.default_rng(seed)
+    x, y = np.arange(nx)[None, :] / nx, np.arange(ny)[:, None] / ny
+    w = [sum(a * np.sin(2 * np.pi * (k * x + m * y) + p) for k, m, a, p in
+             zip(rng.integers(1, 4, 3), rng.integers(0, 3, 3), rng.uniform(0.01, 0.05, 3), rng.uniform(0, 6, 3)))
+         for _ in range(4)]
+    left = x < 0.5
+    return [np.where(left, 1.0, 0.3) * (1 + w[0]), 0.2 + w[1], w[2], np.where(left, 1.1, 0.8) * (1 + w[3])]
+
+
+def _run(nx, ny, bc, prec, variant, power, steps):
+    s = F.Solver(nx, ny, 1e-3, 1e-3, 1e-5, 1e-5, 2.0, bc, prec)
+    s.set_variant(variant)
+    s.set_macro(*_state(nx, ny, nx + ny))
+    s.set_f(s.get_f() * 2.0**power)
+    s.step(steps)
+    assert s.sync() == F.FDLBM_OK
+    f = s.get_f()
+    s.close()
+    return f * 2.0**-power
+
+
+@pytest.mark.parametrize("power", [84, -84, 104])
+@pytest.mark.parametrize("nx,ny,bc,variant", [(61, 9, [OUT, OUT, WALL, WALL], 9), (130, 4, [OUT, OUT, PER, PER], 0),
+                                              (259, 171, [PER] * 4, 0), (11003, 4, [OUT, OUT, PER, PER], 2)])
+def test_fp64_step_at_any_density(nx, ny, bc, variant, power):
+    assert np.array_equal(_run(nx, ny, bc, F.FDLBM_FP64, variant, power, 3),
+                          _run(nx, ny, bc, F.FDLBM_FP64, variant, 0, 3))
