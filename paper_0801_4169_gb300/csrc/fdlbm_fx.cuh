@@ -250,11 +250,11 @@ FX_HD Base base_of(double A0, double A1, double p0, double p1, double p2, double
   if (bits_of(A0) >> 63) b.A0f = -b.A0f;
   return b;
 }
-// A weight nF_k that the fixed-point form can take, for FP64 results: 2^-700 < |nF_k| < 2^700. Its exponent is part of
+// A weight nF_k that the fixed-point form can take. FP64 results: 2^-700 < |nF_k| < 2^700. Its exponent is part of
 // the results' scale alone, an integer; the limits keep the results normal.
 FX_HD bool weight_ok(double nF) { return abs_hi(nF) - ((1023u - 700u) << 20) < 1400u << 20; }
-// ... for FP32 results, whose scale is an FP32 number: 2^-60 < |nF_k| < 2^40
-FX_HD bool weight_ok_f32(double nF) { return abs_hi(nF) - ((1023u - 60u) << 20) < 100u << 20; }
+// ... for FP32 results, in units of 2^ex: those whose scale 2^(ex + 36) beside narrow_f32 is an FP32 number
+FX_HD bool unit_ok_f32(int ex) { return (unsigned)(ex + 36 + 149) <= 149u + 127u; }
 // es of ring k
 FX_HD int scale_of(const Base& b, int k) {
   const float v = k == 0 ? 1.0f : k == 1 ? 1.92f : k == 2 ? 2.99f : 4.49f;
@@ -343,18 +343,19 @@ FX_HD void pair_of(const RingFx& r, const Dir& d, s64& NE, s64& NO) {
   NE = r.A0 + mul2(r.c1, d.q1, r.c2, d.q2, start);
   NO = mul2(r.c3, d.q3, r.c4, d.q4, start);
 }
-// R 2^ex as an FP32 number, |R| < 2^60: R = hi 2^36 + lo 2^4 with hi exact in FP32, so one rounding of
-// R's leading bits (and one of lo, 2^-24 of 2^36 units). up = 2^(ex + 36), down = 2^(ex + 4).
-FX_HD float narrow_f32(s64 R, float up, float down) {
+// R as an FP32 number in units of 2^36, |R| < 2^60: R = hi 2^36 + lo 2^4 with hi exact in FP32, so one rounding of
+// R's leading bits (and one of lo, 2^-24 of 2^36 units). The caller's scale 2^(ex + 36) then changes no bit.
+FX_HD float narrow_f32(s64 R) {
   const int hi = (int)(R >> 32) >> 4;
   const unsigned lo = (unsigned)(R >> 4);
 #ifdef __CUDA_ARCH__
-  return __fmaf_rn(__int2float_rn(hi), up, __fmul_rn(__uint2float_rn(lo), down));
+  return __fmaf_rn(__uint2float_rn(lo), 0x1p-32f, __int2float_rn(hi));
 #else
-  return std::fma((float)hi, up, (float)lo * down);
+  return std::fma((float)lo, 0x1p-32f, (float)hi);
 #endif
 }
-FX_HD float pow2_f32(int e) { return float_of((unsigned)(e + 127) << 23); }
+// 2^e, e in -149..127
+FX_HD float pow2_f32(int e) { return float_of(e >= -126 ? (unsigned)(e + 127) << 23 : 1u << ((e + 149) & 31)); }
 
 }  // namespace fx
 }  // namespace fdlbm

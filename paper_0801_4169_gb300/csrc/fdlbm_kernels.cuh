@@ -727,17 +727,17 @@ __device__ constexpr int dir_minus(int t) { return t == 0 ? 3 : t + 3; }
 // r f_eq of ring K's 8 directions; nF = ring_weight<false>(e, K, c). n..T: the node's macros (rare form).
 __device__ __forceinline__ void feq_ring(const FeqNode& e, int K, double nF, const Coeffs& c, double n, double ux,
                                          double uy, double T, float (&fe)[8]) {
-  if (__builtin_expect(e.b.ok && fx::weight_ok_f32(nF), 1)) {
+  if (__builtin_expect(e.b.ok && fx::unit_ok_f32(e.es + fx::exp_of(fx::abs_hi(nF)) - 62), 1)) {
     const fx::RingFx r = fx::ring_shared(e.A0, e.es, nF, c.fxc[0][K]);
-    const float up = fx::pow2_f32(r.ex + 36), down = fx::pow2_f32(r.ex + 4);
+    const float up = fx::pow2_f32(r.ex + 36);
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       long long NE, NO;
       fx::pair_of<false>(r, e.q[t], NE, NO);
-      const float ev = fx::narrow_f32(NE, up, down);
-      const float od = __uint_as_float(__float_as_uint(fx::narrow_f32(NO, up, down)) ^ ((e.neg >> t) << 31));
-      fe[dir_plus(t)] = ev + od;
-      fe[dir_minus(t)] = ev - od;
+      const float ev = fx::narrow_f32(NE);
+      const float od = fx::narrow_f32(NO) * __uint_as_float(__float_as_uint(up) ^ ((e.neg >> t) << 31));
+      fe[dir_plus(t)] = fmaf(ev, up, od);
+      fe[dir_minus(t)] = fmaf(ev, up, -od);
     }
   } else {
     const F8 o = feq_ring_rare(n, ux, uy, T, K, c);

@@ -42,3 +42,33 @@ def _run(nx, ny, bc, prec, variant, power, steps):
 def test_fp64_step_at_any_density(nx, ny, bc, variant, power):
     assert np.array_equal(_run(nx, ny, bc, F.FDLBM_FP64, variant, power, 3),
                           _run(nx, ny, bc, F.FDLBM_FP64, variant, 0, 3))
+
+
+@pytest.mark.parametrize("power", [84, -72])
+@pytest.mark.parametrize("nx,ny,bc,variant", [(61, 9, [OUT, OUT, WALL, WALL], 9), (131, 77, [PER] * 4, 6),
+                                              (259, 171, [OUT] * 4, 12), (130, 4, [OUT, OUT, PER, PER], 2)])
+def test_fp32_storage_step_at_any_density(nx, ny, bc, variant, power):
+    assert np.array_equal(_run(nx, ny, bc, F.FDLBM_FP32_STORE, variant, power, 3),
+                          _run(nx, ny, bc, F.FDLBM_FP32_STORE, variant, 0, 3))
+
+
+@pytest.mark.parametrize("prec", [F.FDLBM_FP64, F.FDLBM_FP32_STORE])
+def test_a_step_takes_as_long_at_any_density(prec):
+    """FP32 storage rounds most of the forms' differences away, so its form shows in the time: 1.5 times the step at
+    n ~ 1 was what all steps took in FP64 arithmetic, 2.4 the FP64 form out of line."""
+    nx, ny, steps = 1024, 768, 10
+    best = {}
+    for power in (0, 84, -84):
+        s = F.Solver(nx, ny, 1e-3, 1e-3, 1e-5, 1e-5, 2.0, [OUT] * 4, prec)
+        m = _state(nx, ny, 5)
+        s.set_macro(m[0] * 2.0**power, *m[1:])
+        s.step(3)
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        for _ in range(5):
+            a.record()
+            s.step(steps)
+            b.record()
+            torch.cuda.synchronize()
+            best[power] = min(best.get(power, np.inf), a.elapsed_time(b))
+        s.close()
+    assert max(best[84], best[-84]) <= 1.5 * best[0]
