@@ -184,7 +184,7 @@ Coeffs make_coeffs(const fdlbm_config* cfg) {
     for (int i = 0; i < 4; ++i) split(c.Fh[k][i], c.dFh[k][i]);
   }
   // Integer weights of the FP64-storage step: units of 2^-S with the sum of a stencil's |weights| (1 - r
-  // among them) below 2^(58 - S), S at most 59. nu is allowed 0.05 lambda, between 1/32 and 1/8.
+  // among them) below 2^(58 - S) for a nu of 0.05 lambda, between 1/32 and 1/8; S at most 59.
   {
     double most = 0.0;
     for (int k = 0; k < 4; ++k) {
@@ -203,7 +203,10 @@ Coeffs make_coeffs(const fdlbm_config* cfg) {
     const int S = 58 - e < 59 ? 58 - e : 59;
     if (S >= 55) {
       c.xS = S;
-      c.xnu = (std::ldexp(1.0, 58 - S) - most) / 8.5;
+      // The weights' sum, nu eight times among them, may reach 15/16 2^(59 - S): with values below 2^58 the sum of the
+      // products' leading parts is then below 15/16 2^61, with r f_eq (below 2^61) the result below 2^62, and a weight's
+      // leading limb below 2^31. A nu of 1/4 on both axes, where Eq. 17's diffusion turns unstable, mostly lies inside.
+      c.xnu = (0.9375 * std::ldexp(1.0, 59 - S) - most) / 8.5;
       if (c.xnu > 0.5) c.xnu = 0.5;
       // from the speeds' decimals, like the moments and f_eq's brackets: a flux by other speeds than the
       // momentum's would differ from it by 2^-53 of f in every step

@@ -19,7 +19,7 @@
 // class, and a stencil aligns its values to their largest class (mixed_entry); where that one agrees
 // throughout, the integers are the same. So a result depends on the node's nine values, its weights
 // and its f_eq alone, not on the tile: every tile shape gives the same bits.
-// The FP64 form (stencil_f64) is left for values or weights outside the integers' range: infinities, NaN,
+// The FP64 form (stencils_f64) is left for values or weights outside the integers' range: infinities, NaN,
 // exponents beyond 2^+-800, nu above the bound that the weights' scale leaves, weights that do not fit.
 #include "fdlbm_kernels.cuh"
 
@@ -221,17 +221,39 @@ __device__ __forceinline__ Macro quad_macro_fx(const double* __restrict__ f, lon
 }
 
 // ---------------------------------------------------------------------------------------------
-// The FP64 form of one direction's r f_eq, for nodes outside the fixed-point range.
-__device__ __noinline__ double feq_one_f64(double n, double ux, double uy, double T, int K, int d, const Coeffs& c) {
+// The FP64 form of r f_eq of ring K, for nodes outside the fixed-point range: the directions of the mask, into their
+// places in f_new (o: the node's entry of the ring's first plane).
+__device__ __noinline__ void feq_f64(double n, double ux, double uy, double T, int K, unsigned mask, const Coeffs& c,
+                                     double* __restrict__ o, long long plane) {
   EqSite e = eq_site(n, ux, uy, T, c);
   // the weight that the rest velocity's is formed from: another rounding of it would make mass
   e.nF[K] = weight_poly<true>(c.r * n * T, T, K, c);
   const EqRing r = eq_ring(e, K, c);
-  const int t = (d == 7 || d == 3) ? 0 : (d == 0 || d == 4) ? 1 : (d == 1 || d == 5) ? 2 : 3;
-  const double p = t == 0 ? e.p[0] : t == 1 ? e.p[1] : t == 2 ? e.p[2] : e.p[3];
-  double fp, fm;
-  eq_pair(r, p, p * p, fp, fm);
-  return d == dir_plus(t) ? fp : fm;
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    double fp, fm;
+    eq_pair(r, e.p[t], e.x[t], fp, fm);
+    if (mask >> dir_plus(t) & 1u) o[dir_plus(t) * plane] = fp;
+    if (mask >> dir_minus(t) & 1u) o[dir_minus(t) * plane] = fm;
+  }
+}
+
+// The same from the pairs' integers, formed again (q: the lane's powers of the projections, stride between them).
+// Out of line: kept for the slow directions in the ring's loop, they cost all others 4%.
+__device__ __noinline__ void feq_slow(s64 A0f, int es, int e0, int ea, int ep, unsigned neg, int K, double nF,
+                                      unsigned mask, const Coeffs& c, const int4* __restrict__ q, int stride,
+                                      double* __restrict__ o, long long plane) {
+  const fx::RingFx r = fx::ring_scaled(A0f, es, e0, ea, ep, K, nF, c.fxc[1][K]);
+#pragma unroll 1
+  for (int t = 0; t < 4; ++t) {
+    const int4 u = q[2 * t * stride], v = q[(2 * t + 1) * stride];
+    s64 NE, NO;
+    fx::pair_of<true>(r, fx::Dir{{u.x, u.y}, {u.z, u.w}, {v.x, v.y}, {v.z, v.w}}, NE, NO);
+    if (neg >> t & 1u) NO = -NO;
+    const int dp = dir_plus(t), dm = dir_minus(t);
+    if (mask >> dp & 1u) o[dp * plane] = fx::to_f64(NE + NO, r.ex);
+    if (mask >> dm & 1u) o[dm * plane] = fx::to_f64(NE - NO, r.ex);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -366,33 +388,43 @@ __device__ __forceinline__ void stencil_box(Acc& a, int& cl, const int2* __restr
     mac(a, t[Y0 + 2].x - t[Y0 + 3].x, t[Y0 + 2].y - t[Y0 + 3].y, c.xD[1][K][CL][0], c.xD[1][K][CL][1]);
   }
 }
-// The FP64 form of direction d of ring K at one node (p: the node's entry of the plane).
-struct SlowArgs {
-  double n, ux, uy, T, nux, nuy;
-};
+// The FP64 form of Eq. 17 for the directions of the mask of ring K at one node: p and o are the node's entries of the
+// ring's first plane in f and f_new, where o holds the directions' r f_eq. The ring's weights are formed once for all of
+// them: with every direction here a site takes some 450 FP64 operations (1024^2 nodes with nu out of range: 1378 us per
+// step; with f_eq and the weights formed again for each direction 4763, in range 830).
 template <bool COH>
-__device__ __noinline__ double stencil_f64(const double* __restrict__ p, int pitch, int K, int d, const SlowArgs& s,
-                                           const Coeffs& c) {
-  const int xs = dir_xs(d), ys = dir_ys(d), cl = dir_cls(d);
-  const double w0 = (1.0 - c.r) - 2.0 * (s.nux + s.nuy);
-  double acc = fma(w0 - c.C2[K][dir_c2(d)], ldf<COH>(p), feq_one_f64(s.n, s.ux, s.uy, s.T, K, d, c));
-  if (xs == 0) {
-    acc = fma(s.nux, ldf<COH>(p + 1) + ldf<COH>(p - 1), acc);
-  } else {
-    const double P1 = c.W1[0][K][cl] + s.nux, M1 = c.Wm1[0][K][cl] + s.nux;
-    acc = fma(xs > 0 ? P1 : M1, ldf<COH>(p + 1), acc);
-    acc = fma(xs > 0 ? M1 : P1, ldf<COH>(p - 1), acc);
-    acc = fma(xs * c.D[0][K][cl], ldf<COH>(p + 2) - ldf<COH>(p - 2), acc);
+__device__ __noinline__ void stencils_f64(const double* __restrict__ p, double* __restrict__ o, long long plane,
+                                          int pitch, int K, unsigned mask, double nux, double nuy, const Coeffs& c) {
+  const double w0 = (1.0 - c.r) - 2.0 * (nux + nuy);
+  double P1[2][2], M1[2][2];
+#pragma unroll
+  for (int l = 0; l < 2; ++l) {
+    P1[0][l] = c.W1[0][K][l] + nux;
+    M1[0][l] = c.Wm1[0][K][l] + nux;
+    P1[1][l] = c.W1[1][K][l] + nuy;
+    M1[1][l] = c.Wm1[1][K][l] + nuy;
   }
-  if (ys == 0) {
-    acc = fma(s.nuy, ldf<COH>(p + pitch) + ldf<COH>(p - pitch), acc);
-  } else {
-    const double P1 = c.W1[1][K][cl] + s.nuy, M1 = c.Wm1[1][K][cl] + s.nuy;
-    acc = fma(ys > 0 ? P1 : M1, ldf<COH>(p + pitch), acc);
-    acc = fma(ys > 0 ? M1 : P1, ldf<COH>(p - pitch), acc);
-    acc = fma(ys * c.D[1][K][cl], ldf<COH>(p + 2 * pitch) - ldf<COH>(p - 2 * pitch), acc);
+#pragma unroll
+  for (int d = 0; d < 8; ++d, p += plane, o += plane) {
+    if (!(mask >> d & 1u)) continue;
+    const int xs = dir_xs(d), ys = dir_ys(d), cl = dir_cls(d);
+    double acc = fma(w0 - c.C2[K][dir_c2(d)], ldf<COH>(p), *o);
+    if (xs == 0) {
+      acc = fma(nux, ldf<COH>(p + 1) + ldf<COH>(p - 1), acc);
+    } else {
+      acc = fma(xs > 0 ? P1[0][cl] : M1[0][cl], ldf<COH>(p + 1), acc);
+      acc = fma(xs > 0 ? M1[0][cl] : P1[0][cl], ldf<COH>(p - 1), acc);
+      acc = fma(xs * c.D[0][K][cl], ldf<COH>(p + 2) - ldf<COH>(p - 2), acc);
+    }
+    if (ys == 0) {
+      acc = fma(nuy, ldf<COH>(p + pitch) + ldf<COH>(p - pitch), acc);
+    } else {
+      acc = fma(ys > 0 ? P1[1][cl] : M1[1][cl], ldf<COH>(p + pitch), acc);
+      acc = fma(ys > 0 ? M1[1][cl] : P1[1][cl], ldf<COH>(p - pitch), acc);
+      acc = fma(ys * c.D[1][K][cl], ldf<COH>(p + 2 * pitch) - ldf<COH>(p - 2 * pitch), acc);
+    }
+    *o = acc;
   }
-  return acc;
 }
 // The ghost copies that an edge node owns of ring K's velocities, from the values it has just stored.
 __device__ __noinline__ void ghost_ring(double* fn, const Grid& g, int gx, int gy, GhostOwn go, int K) {
@@ -655,7 +687,7 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
       sm.q[(2 * t) * NT + tid] = make_int4(e.q[t].q1.h, e.q[t].q1.l, e.q[t].q2.h, e.q[t].q2.l);
       sm.q[(2 * t + 1) * NT + tid] = make_int4(e.q[t].q3.h, e.q[t].q3.l, e.q[t].q4.h, e.q[t].q4.l);
     }
-    // |nu| <= xnu keeps the weights' sum below 2^58
+    // |nu| <= xnu keeps the weights' sum below 15/16 2^59
     fixed = c.xS != 0 && e.b.ok && fabs(dnux) <= c.xnu && fabs(dnuy) <= c.xnu;
     if (fixed) {
       nuxi = nu_fixed(dnux, c.xS);
@@ -681,12 +713,12 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
     if (!mine) continue;
     const double nF = ring_weight<true>(e, K, c);
     snF += nF;
+    double* o = fn + (long long)(1 + 8 * K) * g.plane + off;
     unsigned slow = 0xffu;  // directions left to the FP64 form
     if (fixed && fx::weight_ok(nF)) {
       slow = 0u;
       const fx::RingFx r = fx::ring_scaled(e.b.A0f, fx::scale_of(e.b, K), e.b.e0, e.b.ea, e.b.ep, K, nF, c.fxc[1][K]);
       const int2* b = &sm.box[0][(ty + 2) * X::BW + tx + 2];
-      double* o = fn + (long long)(1 + 8 * K) * g.plane + off;
       auto powers = [&](int t) {
         const int4 u = sm.q[(2 * t) * NT + tid], v = sm.q[(2 * t + 1) * NT + tid];
         return fx::Dir{{u.x, u.y}, {u.z, u.w}, {v.x, v.y}, {v.z, v.w}};
@@ -716,12 +748,11 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
       else ring(std::true_type{});
     }
     if (slow) {
-      const SlowArgs sa{sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], dnux, dnuy};
-#pragma unroll 1
-      for (int d = 0; d < 8; ++d) {
-        const long long at = (long long)(1 + 8 * K + d) * g.plane + off;
-        if ((slow >> d) & 1u) fn[at] = stencil_f64<COH>(f + at, g.pitch, K, d, sa, c);
-      }
+      if (e.b.ok && fx::weight_ok(nF))
+        feq_slow(e.b.A0f, fx::scale_of(e.b, K), e.b.e0, e.b.ea, e.b.ep, e.neg, K, nF, slow, c, sm.q + tid, NT, o, g.plane);
+      else
+        feq_f64(sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], K, slow, c, o, g.plane);
+      stencils_f64<COH>(f + (o - fn), o, g.plane, g.pitch, K, slow, dnux, dnuy, c);
     }
     if (go.mx | go.my) ghost_ring(fn, g, gx, gy, go, K);
   }
@@ -888,7 +919,7 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
     const double nF = sm.nF[nd][K];
     const int diag = pg & 1;
     const s64 nuxi = sm.nui[nd][0], nuyi = sm.nui[nd][1];
-    const bool fixed = sm.ok[nd] && sm.nufit[nd][0] && sm.nufit[nd][1] && fx::weight_ok(nF);
+    const bool fits = sm.nufit[nd][0] && sm.nufit[nd][1], brackets = sm.ok[nd] && fx::weight_ok(nF);
     const fx::RingFx r = fx::ring_scaled(sm.A0f[nd], sm.es[nd][K], sm.e0[nd], sm.ea[nd], sm.ep[nd], K, nF, c.fxc[1][K]);
     const L28 nux = l28(nuxi), nuy = l28(nuyi);
     const ClassW w = class_w(c, K, diag, nuxi, nuyi);
@@ -903,6 +934,9 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
       s64 NE, NO;
       fx::pair_of<true>(r, fx::Dir{{u.x, u.y}, {u.z, u.w}, {v4.x, v4.y}, {v4.z, v4.w}}, NE, NO);
       if ((sm.neg[nd] >> T) & 1) NO = -NO;
+      if (!brackets)
+        feq_f64(sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], K, 1u << dir_plus(T) | 1u << dir_minus(T), c,
+                fn + (long long)(1 + 8 * K) * g.plane + off, g.plane);
 #pragma unroll 1
       for (int m = 0; m < 2; ++m) {
         const int d = m ? dir_minus(T) : dir_plus(T), q = 1 + 8 * K + d;
@@ -910,7 +944,7 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
         const int2* b = &sm.box[8 * K + d][(ty + 2) * X::BW + tx + 2];
         int cl = sm.cls[8 * K + d];
         int2 t[9] = {b[0], b[ox], b[-ox], b[2 * ox], b[-2 * ox], b[oy], b[-oy], b[2 * oy], b[-2 * oy]};
-        bool ok = fixed && cl != kFar;
+        bool ok = brackets && fits && cl != kFar;
         if (cl & kMixed) {
           // a cell that the direction does not reach has no say in the class
           if (!hx) t[3] = t[4] = t[0];
@@ -928,14 +962,16 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
         mac(a, at(5), Py);
         mac(a, at(6), My);
         mac(a, t[7].x - t[8].x, t[7].y - t[8].y, Dy.h, Dy.l);
+        const s64 B = m ? NE - NO : NE + NO;
         double v;
-        ok = finish(a, m ? NE - NO : NE + NO, r.ex, 4 * cl - 1024 - c.xS, v) && ok;
+        ok = finish(a, B, r.ex, 4 * cl - 1024 - c.xS, v) && ok;
         const long long to = (long long)q * g.plane + off;
+        if (ok || brackets) fn[to] = ok ? v : fx::to_f64(B, r.ex);
         if (!ok) {
-          const SlowArgs sa{sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], sm.nu[nd][0], sm.nu[nd][1]};
-          v = stencil_f64<COH>(f + to, g.pitch, K, d, sa, c);
+          const long long ring = to - d * g.plane;
+          stencils_f64<COH>(f + ring, fn + ring, g.plane, g.pitch, K, 1u << d, sm.nu[nd][0], sm.nu[nd][1], c);
+          v = fn[to];
         }
-        fn[to] = v;
         if (go.mx | go.my) ghost_one(fn, g, gx, gy, go, q, v);
       }
     }
