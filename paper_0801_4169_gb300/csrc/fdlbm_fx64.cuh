@@ -15,12 +15,14 @@
 // (E its biased exponent), its integer V = +-m 2^(E - 4c + 5) with m the 53-bit significand: exact,
 // below 2^58, in units of 2^(4c - 1080). A plane's values are converted once per tile, into shared
 // memory, and the nine values of a stencil combine directly where the tile's classes agree. Where a
-// tile holds several classes of a plane (f crosses a power of 16, or zero) its entries keep their own
-// class, and a stencil aligns its values to their largest class (mixed_entry); where that one agrees
-// throughout, the integers are the same. So a result depends on the node's nine values, its weights
-// and its f_eq alone, not on the tile: every tile shape gives the same bits.
-// The FP64 form (stencils_f64) is left for values or weights outside the integers' range: infinities, NaN,
-// exponents beyond 2^+-800, nu above the bound that the weights' scale leaves, weights that do not fit.
+// tile holds several classes of a plane (f crosses a power of 16, or zero) its cells stay FP64 numbers,
+// and a stencil converts its nine values to their largest class itself (align_cells), rounding what drops
+// out; where that one agrees throughout, the integers are the same. So a result depends on the node's nine
+// values, its weights and its f_eq alone, not on the tile: every tile shape gives the same bits.
+// The integers carry a few units of error whatever the weights are. Where a stencil's values differ by classes, a value
+// that hardly counts can set the unit, so there a result has to have 2^45 units, or the node's density 2^49 of them; the
+// FP64 form (stencils_f64) takes the others' place, as it does for values or weights outside the integers' range:
+// infinities, NaN, exponents beyond 2^+-800, nu above the bound that the weights' scale leaves, weights that do not fit.
 #include "fdlbm_kernels.cuh"
 
 namespace fdlbm {
@@ -246,11 +248,12 @@ __device__ __noinline__ void feq_slow(s64 A0f, int es, int e0, int ea, int ep, u
   const fx::RingFx r = fx::ring_scaled(A0f, es, e0, ea, ep, K, nF, c.fxc[1][K]);
 #pragma unroll 1
   for (int t = 0; t < 4; ++t) {
+    const int dp = dir_plus(t), dm = dir_minus(t);
+    if (!(mask & (1u << dp | 1u << dm))) continue;
     const int4 u = q[2 * t * stride], v = q[(2 * t + 1) * stride];
     s64 NE, NO;
     fx::pair_of<true>(r, fx::Dir{{u.x, u.y}, {u.z, u.w}, {v.x, v.y}, {v.z, v.w}}, NE, NO);
     if (neg >> t & 1u) NO = -NO;
-    const int dp = dir_plus(t), dm = dir_minus(t);
     if (mask >> dp & 1u) o[dp * plane] = fx::to_f64(NE + NO, r.ex);
     if (mask >> dm & 1u) o[dm * plane] = fx::to_f64(NE - NO, r.ex);
   }
@@ -262,8 +265,8 @@ struct L28 {
   int h, l;
 };
 __device__ __forceinline__ L28 l28(s64 v) { return L28{(int)(v >> 28), (int)v & 0xfffffff}; }
-// Marks of a plane's class entry: several classes; the FP64 form (kFar has kMixed's bit)
-constexpr int kMixed = 1 << 16, kFar = -1;
+// A plane's class entry where its cells are FP64 numbers: several classes, or one outside the integer form's range
+constexpr int kMixed = 1 << 16;
 // Class range of the integer form: results and their units stay normal FP64 numbers
 constexpr int kClsMin = 56, kClsMax = 456;
 // A value's integer, m 2^sh with its sign; sh = E - 4c + 5, in 2..5
@@ -317,29 +320,57 @@ __device__ __forceinline__ bool finish(const Acc& a, s64 B, int ex, int unit, do
   return l <= 29 && ((unsigned)(hi ^ (hi >> 31)) >> ((29 - l) & 31)) == 0u && (unsigned)(R >> 32) + 1u > 1u;
 }
 
-// Box entries of a plane with several classes: the value's integer in its own class, and in the four
-// bits above l how many classes it lies below the plane's largest (15 and more: the integer is 0).
-__device__ __forceinline__ int2 mixed_entry(double x, int cl) {
-  const int E = (int)(((unsigned)__double2hiint(x) & 0x7fffffffu) >> 20);
-  const int c = (E + 3) >> 2, below = cl - c;
-  if (below >= 15) return make_int2(0, (int)(15u << 28));
-  const L28 t = l28(val_fixed(x, E - 4 * c + 5));
-  return make_int2(t.h, (int)((unsigned)t.l | (unsigned)below << 28));
-}
-// Nine entries of such a plane to their largest class, which cl (the plane's largest) becomes.
-__device__ __forceinline__ void align_entries(int2 (&t)[9], int& cl) {
-  int least = 15;
+// A plane of several classes: a stencil's first NP cells, FP64 numbers, become integers of their largest class cl,
+// m 2^(6 - s) with s = 4 cl + 1 - E, rounded to nearest even: a rounding of one sign would add up. FP64 numbers in the
+// box and not integers of 15 classes below the plane's largest, since no span of a tile's values may change a stencil's:
+// 1023 x 777 497 us per step against 503, a 32-tube batch 23.0 ms against 23.6, 400 x 4 10.4 us against 10.0.
+template <int NP>
+__device__ __forceinline__ void align_cells(int2 (&t)[9], int& cl) {
+  unsigned top = 0u;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) least = min(least, (int)((unsigned)t[i].y >> 28));
+  for (int i = 0; i < NP; ++i) top = max(top, (unsigned)t[i].y & 0x7fffffffu);
+  cl = ((int)(top >> 20) + 3) >> 2;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const L28 u = l28((((s64)t[i].x << 28) + (t[i].y & 0xfffffff)) >> 4 * ((int)((unsigned)t[i].y >> 28) - least));
+  for (int i = 0; i < NP; ++i) {
+    const unsigned hi = (unsigned)t[i].y, lo = (unsigned)t[i].x, m = (hi & 0xfffffu) | 0x100000u;
+    const int s = min(4 * cl + 1 - (int)((hi & 0x7fffffffu) >> 20), 63);  // 1..; of a zero 63, which leaves nothing
+    const u64 v = ((u64)__funnelshift_l(lo, m, 6) << 32) | (lo << 6);
+    const u64 r = (v + ((1ull << (s - 1)) - 1ull) + ((v >> s) & 1ull)) >> s;
+    const s64 sg = (s64)((int)hi >> 31);
+    const L28 u = l28((s64)(r ^ (u64)sg) - sg);
     t[i] = make_int2(u.h, u.l);
   }
-  cl -= least;
 }
-// Direction D at a node from the converted box (b: the node's entry of the plane, rows of BW). MIXED: the
-// plane holds several classes; the stencil's values enter at their largest class, which cl becomes.
+// Whether a result of a plane of several classes may stay: 2^45 units of 2^unit or more, or the node's n 2^49 units.
+// If not, several_classes looks at the stencil itself. The nodes that this leaves to the FP64 form, one direction in 10^5
+// along a Mach 6 shock and none in smooth flow, cost the double Mach reflection 3% (100.5 -> 103.6 us per step).
+__device__ __forceinline__ bool precise(double out, int unit, double n) {
+  const int e = (int)((unsigned)__double2hiint(out) >> 20 & 0x7ffu) - 1023;
+  return e >= unit + 45 || (int)((unsigned)__double2hiint(n) >> 20) - 1023 >= unit + 49;
+}
+// The directions of the mask, of planes of several classes, whose stencils hold several (b: the node's entry of the ring's
+// first plane, planes BN apart, rows of BW)
+template <int BN, int BW>
+__device__ __noinline__ unsigned several_classes(const int2* __restrict__ b, unsigned mask) {
+  unsigned out = 0u;
+#pragma unroll 1
+  for (int d = 0; d < 8; ++d, b += BN) {
+    if (!(mask >> d & 1u)) continue;
+    const int x2 = dir_xs(d) ? 2 : 1, y2 = dir_ys(d) ? 2 * BW : BW;
+    const int at[9] = {0, 1, -1, x2, -x2, BW, -BW, y2, -y2};
+    int lo = 1 << 20, hi = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int c = ((int)((unsigned)b[at[i]].y >> 20 & 0x7ffu) + 3) >> 2;
+      lo = min(lo, c);
+      hi = max(hi, c);
+    }
+    if (lo != hi) out |= 1u << d;
+  }
+  return out;
+}
+// Direction D at a node from the box (b: the node's entry of the plane, rows of BW). MIXED: the plane may hold several
+// classes; the stencil's values then enter at their largest class, which cl becomes.
 template <int D, int BW, bool MIXED>
 __device__ __forceinline__ void stencil_box(Acc& a, int& cl, const int2* __restrict__ b, const ClassW& w, L28 w0,
                                             const Coeffs& c, int K, L28 nux, L28 nuy) {
@@ -361,15 +392,7 @@ __device__ __forceinline__ void stencil_box(Acc& a, int& cl, const int2* __restr
     t[Y0 + 3] = b[-2 * YS * BW];
   }
   if constexpr (MIXED) {
-    int least = 15;  // as align_entries, for the direction's own cells
-#pragma unroll
-    for (int i = 0; i < NP; ++i) least = min(least, (int)((unsigned)t[i].y >> 28));
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const L28 u = l28((((s64)t[i].x << 28) + (t[i].y & 0xfffffff)) >> 4 * ((int)((unsigned)t[i].y >> 28) - least));
-      t[i] = make_int2(u.h, u.l);
-    }
-    cl -= least;
+    if (cl & kMixed) align_cells<NP>(t, cl);
   }
   auto at = [&](int i) { return L28{t[i].x, t[i].y}; };
   mac(a, at(0), w0);
@@ -414,14 +437,14 @@ __device__ __noinline__ void stencils_f64(const double* __restrict__ p, double* 
     } else {
       acc = fma(xs > 0 ? P1[0][cl] : M1[0][cl], ldf<COH>(p + 1), acc);
       acc = fma(xs > 0 ? M1[0][cl] : P1[0][cl], ldf<COH>(p - 1), acc);
-      acc = fma(xs * c.D[0][K][cl], ldf<COH>(p + 2) - ldf<COH>(p - 2), acc);
+      acc = fma(xs > 0 ? c.D[0][K][cl] : -c.D[0][K][cl], ldf<COH>(p + 2) - ldf<COH>(p - 2), acc);
     }
     if (ys == 0) {
       acc = fma(nuy, ldf<COH>(p + pitch) + ldf<COH>(p - pitch), acc);
     } else {
       acc = fma(ys > 0 ? P1[1][cl] : M1[1][cl], ldf<COH>(p + pitch), acc);
       acc = fma(ys > 0 ? M1[1][cl] : P1[1][cl], ldf<COH>(p - pitch), acc);
-      acc = fma(ys * c.D[1][K][cl], ldf<COH>(p + 2 * pitch) - ldf<COH>(p - 2 * pitch), acc);
+      acc = fma(ys > 0 ? c.D[1][K][cl] : -c.D[1][K][cl], ldf<COH>(p + 2 * pitch) - ldf<COH>(p - 2 * pitch), acc);
     }
     *o = acc;
   }
@@ -496,10 +519,9 @@ struct FxCells {
 
 // One warp converts one plane into its box, from the lane's cells' values v (a cell that no stencil reads
 // takes another cell's value); returns the plane's class entry.
-template <int TW, int TH, bool COH, bool DUP = false>
-__device__ __forceinline__ int convert_plane(const double* __restrict__ pl, const Grid& g, int x0, int y0, int lane,
-                                             const double (&v)[FxCells<TW, TH, DUP>::NV], int2* __restrict__ box) {
-  using X = FxBox<TW, TH>;
+template <int TW, int TH, bool DUP = false>
+__device__ __forceinline__ int convert_plane(int lane, const double (&v)[FxCells<TW, TH, DUP>::NV],
+                                             int2* __restrict__ box) {
   using C = FxCells<TW, TH, DUP>;
   constexpr int NV = C::NV;
   unsigned amax = 0u, amin = 0x7fffffffu;
@@ -511,8 +533,7 @@ __device__ __forceinline__ int convert_plane(const double* __restrict__ pl, cons
   }
   const int cl = ((int)(__reduce_max_sync(0xffffffffu, amax) >> 20) + 3) >> 2;
   const int cm = ((int)(__reduce_min_sync(0xffffffffu, amin) >> 20) + 3) >> 2;
-  if (cl < kClsMin || cl > kClsMax) return kFar;
-  if (cl == cm) {
+  if (cl == cm && cl >= kClsMin && cl <= kClsMax) {
 #pragma unroll
     for (int i = 0; i < NV; ++i) {
       const int2 p = C::cell(lane + 32 * i);
@@ -522,22 +543,12 @@ __device__ __forceinline__ int convert_plane(const double* __restrict__ pl, cons
     }
     return cl;
   }
-  if constexpr (NV <= 4) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int2 p = C::cell(lane + 32 * i);
-      const int2 w = mixed_entry(v[i], cl);
-      if (lane + 32 * i < C::N) C::put(box, p, w);
-    }
-  } else {  // the cells again, in a loop
-#pragma unroll 1
-    for (int i = lane; i < C::N; i += 32) {
-      const int2 p = C::cell(i);
-      if (X::needed(g, x0 + p.x, y0 + p.y))
-        C::put(box, p, mixed_entry(ldf<COH>(pl + (long long)(y0 + p.y) * g.pitch + x0 + p.x), cl));
-    }
+  for (int i = 0; i < NV; ++i) {
+    const int2 p = C::cell(lane + 32 * i);
+    if (lane + 32 * i < C::N) C::put(box, p, make_int2(__double2loint(v[i]), __double2hiint(v[i])));
   }
-  return cl | kMixed;
+  return kMixed;
 }
 template <int TW, int TH, bool DUP = false>
 __device__ __forceinline__ void plane_cells(const Grid& g, int x0, int y0, int lane,
@@ -571,11 +582,12 @@ __device__ __forceinline__ s64 nu_fixed(double nu, int S) {  // nu 2^S, truncate
   return (unsigned)__double2hiint(nu) >> 31 ? -a : a;
 }
 // f_eq and Eq. 17 of the pair of directions T of ring K (box: the node's entry in the ring's first plane,
-// planes BN apart; MIXED: planes of several classes). Returns the mask of directions that did not fit.
+// planes BN apart; MIXED: planes of several classes, n: the node's density). Returns the mask of directions
+// that did not fit, and above it (<< 8) of those that have to be of one class (precise).
 template <int T, int BN, int BW, bool MIXED>
 __device__ __forceinline__ unsigned pair_box(const int2* __restrict__ box, const fx::RingFx& r, const fx::Dir& d,
                                              bool neg, const ClassW& w, L28 w0, L28 nux, L28 nuy, const Coeffs& c,
-                                             int K, const int* __restrict__ cls, double* __restrict__ o,
+                                             int K, double n, const int* __restrict__ cls, double* __restrict__ o,
                                              long long plane) {
   s64 NE, NO;
   fx::pair_of<true>(r, d, NE, NO);
@@ -585,13 +597,13 @@ __device__ __forceinline__ unsigned pair_box(const int2* __restrict__ box, const
   auto one = [&](auto dc, s64 B) {
     constexpr int D = decltype(dc)::value;
     int cl = cls[D];
-    const bool far = MIXED && cl == kFar;
-    if constexpr (MIXED) cl &= ~kMixed;
     Acc a = acc_start(lsum);
     stencil_box<D, BW, MIXED>(a, cl, box + D * BN, w, w0, c, K, nux, nuy);
+    const int unit = 4 * cl - 1024 - c.xS;
     double v;
-    const bool ok = finish(a, B, r.ex, 4 * cl - 1024 - c.xS, v);
-    if (!ok || (MIXED && (far || cl < kClsMin))) bad |= 1u << D;
+    const bool ok = finish(a, B, r.ex, unit, v);
+    if (!ok || (MIXED && (cl < kClsMin || cl > kClsMax))) bad |= 1u << D;
+    if (MIXED && !precise(v, unit, n)) bad |= 0x100u << D;
     o[D * plane] = v;
   };
   one(std::integral_constant<int, dir_plus(T)>{}, NE + NO);
@@ -618,7 +630,7 @@ struct FxTile {
   int4 q[8 * NT];  // fx::Dir of direction t: [2 t][lane] (q1, q2), [2 t + 1][lane] (q3, q4)
   int2 box[8][FxBox<TW, TH>::BN];
   double n[SN], ux[SN], uy[SN], T[SN], P[SN];
-  int cls[8];  // the planes' classes, + kMixed: several; kFar: the FP64 form
+  int cls[8];  // the planes' classes, or kMixed
 };
 
 // One tile of the FP64 step, one lane per node, the rings one after the other. A tile that holds a
@@ -706,7 +718,7 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
       double v[NV];
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = ldf<COH>(pl + src[i]);
-      const int cl = convert_plane<TW, TH, COH, DUP>(pl, g, x0, y0, lane, v, sm.box[q]);
+      const int cl = convert_plane<TW, TH, DUP>(lane, v, sm.box[q]);
       if (lane == 0) sm.cls[q] = cl;
     }
     __syncthreads();
@@ -730,23 +742,26 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
       auto ring = [&](auto mixed) {
         constexpr bool MX = decltype(mixed)::value;
         constexpr int N = X::BN, W = X::BW;
+        const double n = MX ? sm.n[so] : 0.0;
         {
           const ClassW w = class_w(c, K, 0, nuxi, nuyi);
           slow |= pair_box<0, N, W, MX>(b, r, powers(0), e.neg & 1u, w, centre_w(c, K, 0, nuxi, nuyi), nux, nuy, c, K,
-                                        sm.cls, o, g.plane);
+                                        n, sm.cls, o, g.plane);
           slow |= pair_box<2, N, W, MX>(b, r, powers(2), e.neg & 4u, w, centre_w(c, K, 1, nuxi, nuyi), nux, nuy, c, K,
-                                        sm.cls, o, g.plane);
+                                        n, sm.cls, o, g.plane);
         }
         {
           const ClassW w = class_w(c, K, 1, nuxi, nuyi);
           const L28 w0 = centre_w(c, K, 2, nuxi, nuyi);
-          slow |= pair_box<1, N, W, MX>(b, r, powers(1), e.neg & 2u, w, w0, nux, nuy, c, K, sm.cls, o, g.plane);
-          slow |= pair_box<3, N, W, MX>(b, r, powers(3), e.neg & 8u, w, w0, nux, nuy, c, K, sm.cls, o, g.plane);
+          slow |= pair_box<1, N, W, MX>(b, r, powers(1), e.neg & 2u, w, w0, nux, nuy, c, K, n, sm.cls, o, g.plane);
+          slow |= pair_box<3, N, W, MX>(b, r, powers(3), e.neg & 8u, w, w0, nux, nuy, c, K, n, sm.cls, o, g.plane);
         }
       };
       if (__builtin_expect(!(any & kMixed), 1)) ring(std::false_type{});  // CTA-uniform
       else ring(std::true_type{});
     }
+    if (slow >> 8) slow |= several_classes<X::BN, X::BW>(&sm.box[0][(ty + 2) * X::BW + tx + 2], slow >> 8);
+    slow &= 0xffu;
     if (slow) {
       if (e.b.ok && fx::weight_ok(nF))
         feq_slow(e.b.A0f, fx::scale_of(e.b, K), e.b.e0, e.b.ea, e.b.ep, e.neg, K, nF, slow, c, sm.q + tid, NT, o, g.plane);
@@ -853,7 +868,7 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
         for (int i = 0; i < NV; ++i) v[j][i] = ldf<COH>(pl + j * g.plane + src[i]);
 #pragma unroll 1
       for (int j = 0; j < U; ++j) {
-        const int cl = convert_plane<TW, TH, COH>(pl, g, x0, y0, lane, v[0], sm.box[q + j]);
+        const int cl = convert_plane<TW, TH>(lane, v[0], sm.box[q + j]);
         if (lane == 0) sm.cls[q + j] = cl;
 #pragma unroll
         for (int k = 0; k + 1 < U; ++k)
@@ -923,6 +938,7 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
     const fx::RingFx r = fx::ring_scaled(sm.A0f[nd], sm.es[nd][K], sm.e0[nd], sm.ea[nd], sm.ep[nd], K, nF, c.fxc[1][K]);
     const L28 nux = l28(nuxi), nuy = l28(nuyi);
     const ClassW w = class_w(c, K, diag, nuxi, nuyi);
+    unsigned slow = 0u;  // directions left to the FP64 form
 #pragma unroll 1
     for (int T = pg; T < 4; T += 4 / PPT) {  // pairs pg, pg + 2
       const bool hx = T != 2, hy = T != 0;
@@ -934,9 +950,6 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
       s64 NE, NO;
       fx::pair_of<true>(r, fx::Dir{{u.x, u.y}, {u.z, u.w}, {v4.x, v4.y}, {v4.z, v4.w}}, NE, NO);
       if ((sm.neg[nd] >> T) & 1) NO = -NO;
-      if (!brackets)
-        feq_f64(sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], K, 1u << dir_plus(T) | 1u << dir_minus(T), c,
-                fn + (long long)(1 + 8 * K) * g.plane + off, g.plane);
 #pragma unroll 1
       for (int m = 0; m < 2; ++m) {
         const int d = m ? dir_minus(T) : dir_plus(T), q = 1 + 8 * K + d;
@@ -944,14 +957,13 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
         const int2* b = &sm.box[8 * K + d][(ty + 2) * X::BW + tx + 2];
         int cl = sm.cls[8 * K + d];
         int2 t[9] = {b[0], b[ox], b[-ox], b[2 * ox], b[-2 * ox], b[oy], b[-oy], b[2 * oy], b[-2 * oy]};
-        bool ok = brackets && fits && cl != kFar;
+        bool ok = brackets && fits;
         if (cl & kMixed) {
           // a cell that the direction does not reach has no say in the class
           if (!hx) t[3] = t[4] = t[0];
           if (!hy) t[7] = t[8] = t[0];
-          cl &= ~kMixed;
-          align_entries(t, cl);
-          ok = ok && cl >= kClsMin;
+          align_cells<9>(t, cl);
+          ok = ok && cl >= kClsMin && cl <= kClsMax;
         }
         auto at = [&](int i) { return L28{t[i].x, t[i].y}; };
         Acc a = acc_start(w0.l + (Px.l + Mx.l) + (Py.l + My.l));
@@ -963,17 +975,34 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
         mac(a, at(6), My);
         mac(a, t[7].x - t[8].x, t[7].y - t[8].y, Dy.h, Dy.l);
         const s64 B = m ? NE - NO : NE + NO;
+        const int unit = 4 * cl - 1024 - c.xS;
         double v;
-        ok = finish(a, B, r.ex, 4 * cl - 1024 - c.xS, v) && ok;
+        ok = finish(a, B, r.ex, unit, v) && ok;
         const long long to = (long long)q * g.plane + off;
-        if (ok || brackets) fn[to] = ok ? v : fx::to_f64(B, r.ex);
-        if (!ok) {
-          const long long ring = to - d * g.plane;
-          stencils_f64<COH>(f + ring, fn + ring, g.plane, g.pitch, K, 1u << d, sm.nu[nd][0], sm.nu[nd][1], c);
-          v = fn[to];
+        if (ok && (sm.cls[8 * K + d] & kMixed) && !precise(v, unit, sm.n[so]))
+          ok = !several_classes<X::BN, X::BW>(&sm.box[8 * K][(ty + 2) * X::BW + tx + 2], 1u << d);
+        if (!ok) {  // r f_eq's integer waits in the place of the result
+          slow |= 1u << d;
+          v = __longlong_as_double(B);
         }
-        if (go.mx | go.my) ghost_one(fn, g, gx, gy, go, q, v);
+        fn[to] = v;
+        if (ok && (go.mx | go.my)) ghost_one(fn, g, gx, gy, go, q, v);
       }
+    }
+    if (slow) {
+      double* o = fn + (long long)(1 + 8 * K) * g.plane + off;
+      if (brackets) {
+#pragma unroll 1
+        for (int d = 0; d < 8; ++d)
+          if (slow >> d & 1u) o[d * g.plane] = fx::to_f64(__double_as_longlong(o[d * g.plane]), r.ex);
+      } else {
+        feq_f64(sm.n[so], sm.ux[so], sm.uy[so], sm.T[so], K, slow, c, o, g.plane);
+      }
+      stencils_f64<COH>(f + (o - fn), o, g.plane, g.pitch, K, slow, sm.nu[nd][0], sm.nu[nd][1], c);
+      if (go.mx | go.my)
+#pragma unroll 1
+        for (int d = 0; d < 8; ++d)
+          if (slow >> d & 1u) ghost_one(fn, g, gx, gy, go, 1 + 8 * K + d, o[d * g.plane]);
     }
     if (pg == 4 / PPT - 1 && K == 0) {
       const double snF = ((sm.nF[nd][0] + sm.nF[nd][1]) + sm.nF[nd][2]) + sm.nF[nd][3];
