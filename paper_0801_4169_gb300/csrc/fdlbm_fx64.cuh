@@ -154,7 +154,8 @@ __device__ __noinline__ Macro node_macro_f64(const double* __restrict__ f, long 
   }
   return to_macro<1>(combine_rings(ldf<COH>(f + off), S, X, Y, c));
 }
-__device__ __forceinline__ bool mom_range(int emax) { return emax >= kMomEmin && emax < 2047 - 8; }
+// The largest sum, 33 x 449^2 times the largest value, stays below 2^1023: its exponent is written without a check.
+__device__ __forceinline__ bool mom_range(int emax) { return emax >= kMomEmin && emax < 2047 - 25; }
 template <bool COH>
 __device__ __forceinline__ Macro node_macro_fx(const double* __restrict__ f, long long plane, long long off,
                                                const Coeffs& c) {

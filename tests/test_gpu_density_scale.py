@@ -28,12 +28,12 @@ def _run(nx, ny, bc, prec, variant, power, steps):
     s = F.Solver(nx, ny, 1e-3, 1e-3, 1e-5, 1e-5, 2.0, bc, prec)
     s.set_variant(variant)
     s.set_macro(*_state(nx, ny, nx + ny))
-    s.set_f(s.get_f() * 2.0**power)
+    s.set_f(np.ldexp(s.get_f(), power))
     s.step(steps)
     assert s.sync() == F.FDLBM_OK
     f = s.get_f()
     s.close()
-    return f * 2.0**-power
+    return np.ldexp(f, -power)
 
 
 @pytest.mark.parametrize("power", [84, -84, 104])
@@ -72,3 +72,13 @@ def test_a_step_takes_as_long_at_any_density(prec):
             best[power] = min(best.get(power, np.inf), a.elapsed_time(b))
         s.close()
     assert max(best[84], best[-84]) <= 1.5 * best[0]
+
+
+@pytest.mark.parametrize("power", [1004, 1008, 1012, -960])
+@pytest.mark.parametrize("nx,ny,bc,variant", [(61, 9, [OUT, OUT, WALL, WALL], 9), (259, 171, [PER] * 4, 0)])
+def test_fp64_step_near_the_ends_of_the_exponent_range(nx, ny, bc, variant, power):
+    """The moments' integer sums carry 10^4 n and 10^4 sum |v|^2 f, which pass 2^1024 where n and its sums do not. There
+    the step computes in FP64: three steps from sum|f| / n below 10 agree to 1000 x 2^-53 of the largest value each."""
+    f = _run(nx, ny, bc, F.FDLBM_FP64, variant, 0, 3)
+    g = _run(nx, ny, bc, F.FDLBM_FP64, variant, power, 3)
+    assert np.abs(f - g).max() <= 3 * 1000 * 2.0**-53 * np.abs(f).max()
