@@ -161,6 +161,8 @@ FX_HD int floor_log2(unsigned x) {
   return x ? 31 - __builtin_clz(x) : -127;
 #endif
 }
+FX_HD int imax(int a, int b) { return a > b ? a : b; }
+FX_HD int imin(int a, int b) { return a < b ? a : b; }
 // |x| 2^(62 - e), truncated; |x| < 2^e. 0 for zero and far smaller values.
 FX_HD s64 from_f64(double x, int e) {
   const u64 b = bits_of(x);
@@ -169,6 +171,15 @@ FX_HD s64 from_f64(double x, int e) {
   const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b;
   const int s = 1022 + e - E;  // >= 0
   return (s64)((m << 9) >> (s < 63 ? s : 63));
+}
+// ... with its sign, rounded to nearest even; |x| < 2^(e - 1)
+FX_HD s64 from_f64_rn(double x, int e) {
+  const u64 b = bits_of(x);
+  const unsigned hi = (unsigned)(b >> 32) & 0x7fffffffu;
+  const u64 m = ((u64)((hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)b, v = m << 9;
+  const int s = imin(1022 + e - (int)(hi >> 20), 63);  // >= 1; of a zero 63, which leaves nothing
+  const u64 r = (v + ((1ull << (s - 1)) - 1ull) + ((v >> s) & 1ull)) >> s;
+  return b >> 63 ? -(s64)r : (s64)r;
 }
 // e with |x| < 2^e (x normal)
 FX_HD int exp_of(unsigned abs_hi_word) { return (int)(abs_hi_word >> 20) - 1022; }
@@ -217,8 +228,6 @@ FX_HD constexpr int exp_c1(int k) { return k == 0 ? 0 : k == 1 ? 2 : k == 2 ? 3 
 FX_HD constexpr int exp_c2(int k) { return k == 0 ? -4 : k == 1 ? 0 : k == 2 ? 2 : 5; }
 FX_HD constexpr int exp_c3(int k) { return k == 0 ? 1 : k == 1 ? 2 : k == 2 ? 2 : 3; }
 FX_HD constexpr int exp_c4(int k) { return k == 0 ? -2 : k == 1 ? 1 : k == 2 ? 3 : 5; }
-FX_HD int imax(int a, int b) { return a > b ? a : b; }
-FX_HD int imin(int a, int b) { return a < b ? a : b; }
 FX_HD unsigned umax(unsigned a, unsigned b) { return a > b ? a : b; }
 // an FP32 number at or just above |x| from its FP64 high word (|x| in the FP32 normal range)
 FX_HD float f32_above(unsigned ah) { return float_of(((ah - (896u << 20)) << 3) + 8u); }

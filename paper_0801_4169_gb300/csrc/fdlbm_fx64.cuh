@@ -578,10 +578,8 @@ __device__ __forceinline__ double axis_nu(double P0, double Pp, double Pm, doubl
   kappa = kappa || ak > 1.0;
   return g.flags & F_NO_VISC ? 0.0 : 0.5 * th * ak * (1.0 - ak);
 }
-__device__ __forceinline__ s64 nu_fixed(double nu, int S) {  // nu 2^S, truncated
-  const s64 a = fx::from_f64(nu, 62 - S);
-  return (unsigned)__double2hiint(nu) >> 31 ? -a : a;
-}
+// nu 2^S to nearest: truncated, the viscosity would be low by half a unit in every step
+__device__ __forceinline__ s64 nu_fixed(double nu, int S) { return fx::from_f64_rn(nu, 62 - S); }
 // f_eq and Eq. 17 of the pair of directions T of ring K (box: the node's entry in the ring's first plane,
 // planes BN apart; MIXED: planes of several classes, n: the node's density). Returns the mask of directions
 // that did not fit, and above it (<< 8) of those that have to be of one class (precise).
