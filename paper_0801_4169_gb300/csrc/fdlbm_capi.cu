@@ -66,6 +66,9 @@ bool valid_cfg(const fdlbm_config* c, std::string* why) {
   return true;
 }
 
+// Grids that the split variants take
+bool split_size(const fdlbm_config* c) { return (long long)c->nx * c->ny > 65536; }
+
 Layout layout_of(const fdlbm_config* c) {
   Layout L;
   L.g.nx = c->nx;
@@ -85,9 +88,10 @@ Layout layout_of(const fdlbm_config* c) {
   L.health_off = 2 * L.fbytes;
   L.stage_off = L.health_off + 256;
   L.mom_off = L.stage_off + round_up((size_t)4 * c->nx * c->ny * sizeof(double), 256);
-  // moment buffer of the split step: 4 FP64 planes + P in the storage precision (the strict step
-  // always goes through it)
-  L.mom_bytes = ((long long)c->nx * c->ny > 65536 && c->prec != FDLBM_FNEQ32) || c->prec == FDLBM_FP64_STRICT
+  // moment buffer of the split step: 4 FP64 planes + P in the storage precision (the strict step always goes through
+  // it; with FP64 storage the split variants are the fused step and need none)
+  const bool split = (c->prec == FDLBM_FP32_STORE || c->prec == FDLBM_FP32_STORE_DW) && split_size(c);
+  L.mom_bytes = split || c->prec == FDLBM_FP64_STRICT
                     ? round_up((size_t)L.g.plane * (4 * sizeof(double) + L.esize), 256) : 0;
   L.total = L.mom_off + L.mom_bytes;
   L.g.mom = nullptr;  // set to the handle's buffer once its memory is known
@@ -315,6 +319,8 @@ int enqueue_health_copy(fdlbm_ctx* h) {
   return FDLBM_OK;
 }
 
+// The split variants' sizes; with FP64 storage, whose split variants are the fused step, the same ones
+bool split_ok(const fdlbm_ctx* h) { return h->grid.mom || (h->cfg.prec == FDLBM_FP64 && split_size(&h->cfg)); }
 bool any_segment(const fdlbm_ctx* h) { return h->seg_on[0] || h->seg_on[1] || h->seg_on[2] || h->seg_on[3]; }
 
 // V_GRP8x4 applies (else its steps are launched one by one as V_RP8x4).
@@ -855,7 +861,7 @@ int fdlbm_variant_count(void) { return V_COUNT; }
 int fdlbm_set_variant(fdlbm_t h, int variant) {
   if (!h) return fail(nullptr, FDLBM_E_ARG, "handle is NULL");
   if (variant < 0 || variant >= V_COUNT) return fail(h, FDLBM_E_ARG, "variant out of range");
-  if (variant_needs_mom(variant) && !h->grid.mom)
+  if (variant_needs_mom(variant) && !split_ok(h))
     return fail(h, FDLBM_E_ARG, "the split variants need a moment buffer, which grids of up to 65536 sites do not have");
   h->variant = variant;
   return FDLBM_OK;
@@ -905,7 +911,7 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
     }
   }
   for (int v = 0; v < V_COUNT && e == cudaSuccess; ++v) {
-    if ((variant_needs_mom(v) && !h->grid.mom) || ((variant_persistent(v) || variant_graph(v)) && !persist_ok)) {
+    if ((variant_needs_mom(v) && !split_ok(h)) || ((variant_persistent(v) || variant_graph(v)) && !persist_ok)) {
       if (times_ms) times_ms[v] = 0.f;  // not available here
       continue;
     }
