@@ -57,10 +57,13 @@ TRAFFIC_B_PER_SITE = {("fp32", 2): 268.5, ("fp32", 6): 267.6, ("fp32", 11): 467.
                       ("fp32dw", 6): 266.3, ("fp32dw", 12): 263.1}
 # Warp instructions issued per site update (ncu smsp__inst_executed over the sites, 2048^2; fp64 1024^2), by
 # (precision, tile variant): these steps bind on instruction issue, whose peak is 4 warp instructions per
-# clock per SM (one per scheduler). FP64 storage serves variants 2, 4-7, 10 and 11 with one kernel.
+# clock per SM (one per scheduler). FP64 storage serves variants 2, 4-7, 10 and 11 with one kernel (32 x 8 tiles), and
+# grids of up to F64_SMALL_SITES sites with the small tiles, which were not counted.
 WARP_INST_PER_SITE = {("fp32", 12): 138.0, ("fp32dw", 6): 131.3, ("fp32dw", 12): 125.0}
 WARP_INST_PER_SITE.update({("fp64", v): 324.3 for v in (2, 4, 5, 6, 7, 10, 11)})
 ISSUE_PER_CLK_SM = 4.0
+F64_SMALL_SITES = 40960
+F64_SMALL_VARIANTS = (3, 8, 9)  # the small tiles at any size
 DTYPE = {"fp64": "f64", "fp32": "f32-store/fixed-point+f64-moments/fixed-point-feq",
          "fneq32": "f64-macros+f32-fneq/f64-step", "fp32dw": "f32-store/df32-feq"}
 # Variants that split a step into two launches (moment pass + update pass; FP64 storage runs its fused step). Their minimum bytes per
@@ -302,11 +305,29 @@ def host_copy_rates(torch, h_src, h_dst):
     return out
 
 
-def issue_roofline(prec_name, variant, site_rate, sm_mhz):
-    """Instruction issue against its peak, where ncu's warp-instruction count for the variant is
+def step_kernel(prec_name, variant, sites):
+    """Name of the kernel that one step of a solve launches."""
+    if prec_name == "fneq32":
+        return "k_step_fneq (FNEQ32 step)"
+    if variant in SPLIT_VARIANTS and prec_name != "fp64":
+        return "k_moments + k_update (split step)"
+    if variant == 12 and prec_name in ("fp32", "fp32dw"):
+        return "k_step_tma (fused step, tile by tensor copy)"
+    if variant in PERSISTENT_VARIANTS and prec_name in ("fp32", "fp64"):
+        return "k_persist_* (persistent steps)"
+    if variant == GRAPH_VARIANT and prec_name in ("fp32", "fp64"):
+        return "small-grid steps replayed from CUDA graphs of 32"
+    if prec_name != "fp64":
+        return "k_step (fused step)"
+    small = sites <= F64_SMALL_SITES or variant in F64_SMALL_VARIANTS
+    return "k_step_fx_small (small tiles, fixed point)" if small else "k_step_fx (fused step, fixed point)"
+
+
+def issue_roofline(prec_name, variant, sites, site_rate, sm_mhz):
+    """Instruction issue against its peak, where ncu's warp-instruction count of the kernel that runs is
     known (else null)."""
     ips = WARP_INST_PER_SITE.get((prec_name, variant))
-    if ips is None:
+    if ips is None or (prec_name == "fp64" and sites <= F64_SMALL_SITES):
         return None
     peak = ISSUE_PER_CLK_SM * N_SM * sm_mhz * 1e6 / 1e9
     achieved = ips * site_rate / 1e9
@@ -344,7 +365,7 @@ def df32_leg(F, torch, w, peaks, sm_mhz, steps=20, warmup=3):
             "autotune_ms": [round(t, 4) for t in times], "status": status,
             "fp64_pipe": {"achieved": fp64, "peak": fp64_peak, "unit": "G FP64-pipe ops/s", "frac": fp64 / fp64_peak},
             "hbm": {"achieved_gbs": hbm, "peak_gbs": peaks.get("hbm_gbs"), "frac": hbm / peaks.get("hbm_gbs", 6800.0)},
-            "issue": issue_roofline("fp32dw", variant, site_rate, sm_mhz),
+            "issue": issue_roofline("fp32dw", variant, w.nx * w.ny, site_rate, sm_mhz),
             "traffic": (TRAFFIC_B_PER_SITE.get(("fp32dw", variant), 0) * w.nx * w.ny or None)
             if (w.nx, w.ny) == (4096, 4096) else None,
             "error_vs_fp64_path": "4096^2, 2000 steps, seeds 0-2: L1(rho) 1.81e-7, 4.32e-7, 8.71e-7 and "
@@ -635,7 +656,7 @@ def main():
     hbm_gbs = (BYTES_PER_LUP_SPLIT if split else BYTES_PER_LUP)[prec_name] * site_rate / 1e9
     tb = TRAFFIC_B_PER_SITE.get((prec_name, variant)) if (w.nx, w.ny) == (4096, 4096) else None
     traffic = tb * w.nx * w.ny if tb else None
-    issue = issue_roofline(prec_name, variant, site_rate, sm_mhz)
+    issue = issue_roofline(prec_name, variant, w.nx * w.ny, site_rate, sm_mhz)
     fp64_pipe = {
         "achieved": achieved, "peak": fp64_peak, "unit": "G FP64-pipe ops/s", "frac": achieved / fp64_peak,
         "peak_derivation": "2 FP64 ops/clk/SM (nominal 1.25 TFLOP/s) x 152 SMs x %.0f MHz sampled" % sm_mhz,
@@ -654,14 +675,7 @@ def main():
                    "l2": "inputs larger than L2 (f pair %.2f GB)" % (BYTES_PER_LUP[prec_name] * w.nx * w.ny / 1e9)
                    if w.nx * w.ny * 33 * 4 > 129e6 else "inputs smaller than L2: steps read a warm cache",
                    "status": status, "parallelism": "replicas%d" % world},
-        "roofline": {"bound": "alu", "kernel": "k_step_fneq (FNEQ32 step)" if prec_name == "fneq32" else
-                     "k_moments + k_update (split step)" if split else
-                     "k_step_tma (fused step, tile by tensor copy)" if variant == 12 and prec_name in ("fp32", "fp32dw")
-                     else "k_persist_* (persistent steps)" if variant in PERSISTENT_VARIANTS
-                     and prec_name in ("fp32", "fp64")
-                     else "small-grid steps replayed from CUDA graphs of 32" if variant == GRAPH_VARIANT
-                     and prec_name in ("fp32", "fp64") else "k_step_fx (fused step, fixed point)"
-                     if prec_name == "fp64" else "k_step (fused step)",
+        "roofline": {"bound": "alu", "kernel": step_kernel(prec_name, variant, w.nx * w.ny),
                      **{k: (issue or fp64_pipe)[k] for k in ("achieved", "peak", "unit", "frac", "peak_derivation")},
                      "traffic": traffic, "traffic_unit": "bytes per step (ncu DRAM read + write of its launches)",
                      "fp64_pipe": fp64_pipe,
