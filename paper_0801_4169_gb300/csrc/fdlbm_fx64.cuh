@@ -602,7 +602,7 @@ __device__ __forceinline__ unsigned pair_box(const int2* __restrict__ box, const
     double v;
     const bool ok = finish(a, B, r.ex, unit, v);
     if (!ok || (MIXED && (cl < kClsMin || cl > kClsMax))) bad |= 1u << D;
-    if (MIXED && !precise(v, unit, n)) bad |= 0x100u << D;
+    if (MIXED && (cls[D] & kMixed) && !precise(v, unit, n)) bad |= 0x100u << D;
     o[D * plane] = v;
   };
   one(std::integral_constant<int, dir_plus(T)>{}, NE + NO);
