@@ -328,10 +328,17 @@ int fdlbm_batch_autotune(fdlbm_batch_t b, int trial_steps, float* times_ms) {
   if (e == cudaSuccess) e = cudaEventCreate(&a1);
   if (e != cudaSuccess) return bcuda(b, e, "autotune events");
   int best = b->variant;
-  float best_ms = 1e30f;
+  float best_ms = 1e30f, timed[V_COUNT] = {};
   for (int v = 0; v < V_COUNT && e == cudaSuccess; ++v) {
     if (!variant_ok(b, v)) {  // ring-parallel variants are single-solve only; FNEQ32 has two shapes
       if (times_ms) times_ms[v] = 0.f;
+      continue;
+    }
+    int twin = 0;  // variants that run one kernel are timed once
+    while (twin < v && !(timed[twin] > 0.f && batch_kernel(b->scheme.prec, twin) == batch_kernel(b->scheme.prec, v))) ++twin;
+    if (twin < v) {
+      timed[v] = timed[twin];
+      if (times_ms) times_ms[v] = timed[v];
       continue;
     }
     b->variant = v;
@@ -352,6 +359,7 @@ int fdlbm_batch_autotune(fdlbm_batch_t b, int trial_steps, float* times_ms) {
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a0, a1);
     ms /= trial_steps;
+    timed[v] = ms;
     if (times_ms) times_ms[v] = ms;
     if (e == cudaSuccess && ms < best_ms) {
       best_ms = ms;

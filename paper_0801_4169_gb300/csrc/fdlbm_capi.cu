@@ -891,7 +891,8 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
   // On small grids the trials advance the state, from a snapshot of the current buffer and health
   // word restored after each variant: the persistent variants (timed there only, where they can
   // win) over their launch, the one-step variants by alternating the buffers as fdlbm_step does.
-  const bool small = (long long)h->cfg.nx * h->cfg.ny <= 262144;
+  const long long sites = (long long)h->cfg.nx * h->cfg.ny;
+  const bool small = sites <= 262144;
   const bool persist_ok = (h->cfg.prec == FDLBM_FP64 || h->cfg.prec == FDLBM_FP32_STORE) && !any_segment(h) && small;
   // Small grids step in tens of microseconds: a few trial steps would weigh the persistent launch's
   // fixed start-up against back-to-back one-step launches, so every variant is timed over at least
@@ -910,9 +911,26 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
       return cuda_fail(h, e, "autotune snapshot");
     }
   }
+  // variants that run one kernel are timed once, and the first of them stands for all: their order by time is noise
+  float timed[V_COUNT] = {};
+  auto keep = [&](int v, float ms) {
+    timed[v] = ms;
+    if (times_ms) times_ms[v] = ms;
+    if (e == cudaSuccess && ms < best_ms) {
+      best_ms = ms;
+      best = v;
+    }
+  };
   for (int v = 0; v < V_COUNT && e == cudaSuccess; ++v) {
     if ((variant_needs_mom(v) && !split_ok(h)) || ((variant_persistent(v) || variant_graph(v)) && !persist_ok)) {
       if (times_ms) times_ms[v] = 0.f;  // not available here
+      continue;
+    }
+    int twin = 0;
+    while (twin < v && !(timed[twin] > 0.f && variant_kernel(h->cfg.prec, twin, sites) == variant_kernel(h->cfg.prec, v, sites)))
+      ++twin;
+    if (twin < v) {
+      keep(v, timed[twin]);
       continue;
     }
     if (variant_graph(v)) {  // replays from the current buffer (each ends there), then the snapshot
@@ -934,11 +952,7 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
       float ms = 0.f;
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
       ms /= (float)replays * kGraphSteps;
-      if (times_ms) times_ms[v] = ms;
-      if (e == cudaSuccess && ms < best_ms) {
-        best_ms = ms;
-        best = v;
-      }
+      keep(v, ms);
       continue;
     }
     if (variant_persistent(v)) {
@@ -956,11 +970,7 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
       float ms = 0.f;
       if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
       ms /= tsteps;
-      if (times_ms) times_ms[v] = ms;
-      if (e == cudaSuccess && ms < best_ms) {
-        best_ms = ms;
-        best = v;
-      }
+      keep(v, ms);
       continue;
     }
     // warm-up launch, then the timed ones. With the snapshot (small grids) they step like
@@ -982,11 +992,7 @@ int fdlbm_autotune(fdlbm_t h, int trial_steps, float* times_ms) {
     float ms = 0.f;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
     ms /= tsteps;
-    if (times_ms) times_ms[v] = ms;
-    if (e == cudaSuccess && ms < best_ms) {
-      best_ms = ms;
-      best = v;
-    }
+    keep(v, ms);
   }
   if (snap) {  // whatever happened above, the state goes back to the snapshot
     cudaError_t e2 = cudaMemcpyAsync(h->f[h->cur], snap, h->fbytes, cudaMemcpyDeviceToDevice, h->stream);

@@ -154,6 +154,14 @@ inline void batch_tile(int prec, int v, int* tw, int* th) {
 
 // FP64 storage: grids up to this many sites run the small tiles whatever the variant (fdlbm_step_f64.cu).
 constexpr long long kF64SmallSites = 40960;
+// The variant that stands for the kernel and shape v runs in a solve: FP64 storage has fewer than variants.
+inline int variant_kernel(int prec, int v, long long sites) {
+  if (prec != FDLBM_FP64 || v == V_RP8x4 || variant_persistent(v) || variant_graph(v)) return v;
+  if (v == V_RP16x4 || v == V_T16x4 || sites <= kF64SmallSites) return V_RP16x4;
+  return v == V_T32x4 ? v : v == V_T32x8 || v == V_TMA32x8 ? V_T32x8 : V_T32x16;
+}
+// ... and in a batch
+inline int batch_kernel(int prec, int v) { return prec == FDLBM_FP64 && v != V_T32x4 ? V_T32x16 : v; }
 constexpr int kPersistMaxSteps = 4096;
 constexpr int kGraphSteps = 32;  // launches per captured graph (even: a replay ends in its first buffer)
 // fdlbm_autotune times every variant over at least this many steps on grids of up to 262144 sites.

@@ -63,21 +63,22 @@ cudaError_t launch_batch_fx(const BatchMember* mem, int nmem, long long n, unsig
 // tile instead; at 333 x 333 it is 121 against 94.
 cudaError_t launch_step_f64(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
                           cudaStream_t s) {
-  if (variant == V_RP8x4) return launch_fx_small<4, 4, 1, 2>(f, fn, g, c, health, s);
-  if (variant == V_RP16x4 || variant == V_T16x4 || (long long)g.nx * g.ny <= kF64SmallSites)
-    return launch_fx_small<8, 4, 2, 4>(f, fn, g, c, health, s);
-  if (variant == V_T32x4) return launch_fx<32, 4, 4>(f, fn, g, c, health, s);
-  if (variant == V_T32x8) return launch_fx<32, 8, 3>(f, fn, g, c, health, s);
-  return launch_fx<32, 8, 2>(f, fn, g, c, health, s);
+  switch (variant_kernel(FDLBM_FP64, variant, (long long)g.nx * g.ny)) {
+    case V_RP8x4: return launch_fx_small<4, 4, 1, 2>(f, fn, g, c, health, s);
+    case V_RP16x4: return launch_fx_small<8, 4, 2, 4>(f, fn, g, c, health, s);
+    case V_T32x4: return launch_fx<32, 4, 4>(f, fn, g, c, health, s);
+    case V_T32x8: return launch_fx<32, 8, 3>(f, fn, g, c, health, s);
+    default: return launch_fx<32, 8, 2>(f, fn, g, c, health, s);
+  }
 }
 
 cudaError_t prepare_batch_f64(int variant) {
-  return variant == V_T32x4 ? prepare_batch_t<32, 4, 4>() : prepare_batch_t<32, 8, 2>();
+  return batch_kernel(FDLBM_FP64, variant) == V_T32x4 ? prepare_batch_t<32, 4, 4>() : prepare_batch_t<32, 8, 2>();
 }
 cudaError_t launch_batch_f64(int variant, const BatchMember* mem, int nmem, long long n, unsigned long long step,
                              const Coeffs& c, cudaStream_t s) {
-  return variant == V_T32x4 ? launch_batch_fx<32, 4, 4>(mem, nmem, n, step, c, s)
-                            : launch_batch_fx<32, 8, 2>(mem, nmem, n, step, c, s);
+  return batch_kernel(FDLBM_FP64, variant) == V_T32x4 ? launch_batch_fx<32, 4, 4>(mem, nmem, n, step, c, s)
+                                                      : launch_batch_fx<32, 8, 2>(mem, nmem, n, step, c, s);
 }
 
 }  // namespace fdlbm
