@@ -578,8 +578,16 @@ __device__ __forceinline__ double axis_nu(double P0, double Pp, double Pm, doubl
   kappa = kappa || ak > 1.0;
   return g.flags & F_NO_VISC ? 0.0 : 0.5 * th * ak * (1.0 - ak);
 }
-// nu 2^S to nearest: truncated, the viscosity would be low by half a unit in every step
-__device__ __forceinline__ s64 nu_fixed(double nu, int S) { return fx::from_f64_rn(nu, 62 - S); }
+// nu in the integer weights' units, where it fits them, and nu the number that the integer stands for: the rest velocity
+// and the FP64 form take that one, since two roundings of nu at a node would make mass. To nearest: truncated, the
+// viscosity would be low by half a unit in every step.
+__device__ __forceinline__ bool nu_fixed(double& nu, const Coeffs& c, s64& nui) {
+  nui = 0;
+  if (!(c.xS != 0 && fabs(nu) <= c.xnu)) return false;
+  nui = fx::from_f64_rn(nu, 62 - c.xS);
+  nu = fx::to_f64(nui, -c.xS);  // exact: of 53 bits or fewer, like nu
+  return true;
+}
 // f_eq and Eq. 17 of the pair of directions T of ring K (box: the node's entry in the ring's first plane,
 // planes BN apart; MIXED: planes of several classes, n: the node's density). Returns the mask of directions
 // that did not fit, and above it (<< 8) of those that have to be of one class (precise).
@@ -699,11 +707,8 @@ __device__ __forceinline__ void fx_tile_body(const double* __restrict__ f, doubl
       sm.q[(2 * t + 1) * NT + tid] = make_int4(e.q[t].q3.h, e.q[t].q3.l, e.q[t].q4.h, e.q[t].q4.l);
     }
     // |nu| <= xnu keeps the weights' sum below 15/16 2^59
-    fixed = c.xS != 0 && e.b.ok && fabs(dnux) <= c.xnu && fabs(dnuy) <= c.xnu;
-    if (fixed) {
-      nuxi = nu_fixed(dnux, c.xS);
-      nuyi = nu_fixed(dnuy, c.xS);
-    }
+    fixed = nu_fixed(dnux, c, nuxi);
+    fixed = nu_fixed(dnuy, c, nuyi) && fixed && e.b.ok;
   }
   constexpr int NV = FxCells<TW, TH, DUP>::NV;
   int src[NV];
@@ -906,12 +911,12 @@ __device__ __forceinline__ void fx_small_tile(const double* __restrict__ f, doub
       } else if (kind == 1) {  // nu along x or y
         bool kappa = false;
         const int step = h ? SW : 1;
-        const double nu = axis_nu(sm.P[so], sm.P[so + step], sm.P[so - step], h ? uy : ux, h ? c.ky : c.kx, g, c, kappa);
+        double nu = axis_nu(sm.P[so], sm.P[so + step], sm.P[so - step], h ? uy : ux, h ? c.ky : c.kx, g, c, kappa);
         if (kappa) bits |= H_KAPPA;
-        const bool fits = c.xS != 0 && fabs(nu) <= c.xnu;
+        s64 nui;
+        sm.nufit[nd][h] = nu_fixed(nu, c, nui);
         sm.nu[nd][h] = nu;
-        sm.nufit[nd][h] = fits;
-        sm.nui[nd][h] = fits ? nu_fixed(nu, c.xS) : 0;
+        sm.nui[nd][h] = nui;
       } else {  // r n F_k of two rings
         const double rnth = c.r * n * T;
         sm.nF[nd][2 * h] = weight_poly<true>(rnth, T, 2 * h, c);
