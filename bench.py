@@ -59,8 +59,8 @@ TRAFFIC_B_PER_SITE = {("fp32", 2): 268.5, ("fp32", 6): 267.6, ("fp32", 11): 467.
 # (precision, tile variant): these steps bind on instruction issue, whose peak is 4 warp instructions per
 # clock per SM (one per scheduler). FP64 storage serves variants 2, 4-7, 10 and 11 with one kernel (32 x 8 tiles), and
 # grids of up to F64_SMALL_SITES sites with the small tiles, which were not counted.
-WARP_INST_PER_SITE = {("fp32", 12): 138.0, ("fp32dw", 6): 131.3, ("fp32dw", 12): 125.0}
-WARP_INST_PER_SITE.update({("fp64", v): 324.3 for v in (2, 4, 5, 6, 7, 10, 11)})
+WARP_INST_PER_SITE = {("fp32", 12): 138.4, ("fp32dw", 6): 131.3, ("fp32dw", 12): 125.0}
+WARP_INST_PER_SITE.update({("fp64", v): 335.3 for v in (2, 4, 5, 6, 7, 10, 11)})
 ISSUE_PER_CLK_SM = 4.0
 F64_SMALL_SITES = 40960
 F64_SMALL_VARIANTS = (3, 8, 9)  # the small tiles at any size

@@ -74,9 +74,11 @@ enum fdlbm_bc { FDLBM_BC_PERIODIC = 0, FDLBM_BC_OUTFLOW = 1, FDLBM_BC_DIRICHLET 
 enum fdlbm_side { FDLBM_LEFT = 0, FDLBM_RIGHT = 1, FDLBM_BOTTOM = 2, FDLBM_TOP = 3 };
 
 /* Storage / arithmetic precision.
- *  FP64        f stored in FP64; moments, f_eq and the stencil in FP64.
- *  FP32_STORE  f stored and differenced in FP32; moments (Eqs. 3-5), weights and
- *              f_eq (Eqs. 10-13) evaluated in FP64. Its rounding error is about
+ *  FP64        f stored in FP64. Moments, f_eq and the stencil are sums of 55 to 62-bit integers where a
+ *              node's numbers allow it, each rounded to FP64 once, and FP64 elsewhere; the macros, the
+ *              weights F_k and nu are formed in FP64.
+ *  FP32_STORE  f stored and differenced in FP32; moments (Eqs. 3-5) and weights evaluated in FP64, f_eq
+ *              (Eqs. 10-13) in 62-bit fixed point (FP64 outside its range). Its rounding error is about
  *              kappa * 2^-24 * n per step, kappa = sum |f_eq| / n, which destroys the
  *              temperature at high Mach number (kappa ~ 1e4 - 1e9).
  *  FNEQ32      f stored as its departure from the local equilibrium: per node the macros
@@ -85,7 +87,8 @@ enum fdlbm_side { FDLBM_LEFT = 0, FDLBM_RIGHT = 1, FDLBM_BOTTOM = 2, FDLBM_TOP =
  *              FP64, takes the new moments (Eqs. 3-5) in FP64 and stores the new g. The
  *              rounding error is then 2^-24 |g| instead of 2^-24 |f|: small where the flow is
  *              near equilibrium, at any Mach number. 164 bytes per node and buffer, against
- *              264 (FP64) and 132 (FP32_STORE); about 1.6x the FP64 path's FP64 work.
+ *              264 (FP64) and 132 (FP32_STORE). Its 927 FP64 operations per site make it the slowest of
+ *              the fast paths: 1000 x 1000 takes 1.86 ms per step, with FP64 0.64.
  *              fdlbm_get_macro returns the stored macros; fdlbm_get_f returns f_eq + g;
  *              fdlbm_set_f stores the FP64 moments of the given f and its departure from their
  *              equilibrium. Batches of FNEQ32 solves take the 32x4 or 32x8 tile variant. */
@@ -105,9 +108,9 @@ enum fdlbm_prec { FDLBM_FP64 = 0, FDLBM_FP32_STORE = 1, FDLBM_FNEQ32 = 2, FDLBM_
  *              operation at a time, with no fused multiply-add, no reassociation and true divisions.
  *              Any IEEE FP64 program taking the same operations in the same order (the order is
  *              spelled out in csrc/fdlbm_strict.cu) gets the same bits; FDLBM_FP64 agrees with it to
- *              rounding (1e-12 relative on smooth flows). It is the slow reference-grade path: 8-9x
- *              the FP64 path's time per step (0.10 GLUPS). One kernel pair: the tile variants do not apply
- *              (fdlbm_set_variant is accepted and ignored; fdlbm_autotune times nothing). Not
+ *              rounding (1e-12 relative on smooth flows). It is the slow reference-grade path
+ *              (300 x 75: 150 us per step, with FP64 40; 2048 x 2048: 22 ms, with FP64 2.4). One
+ *              kernel pair: the tile variants do not apply (fdlbm_set_variant is accepted and ignored; fdlbm_autotune times nothing). Not
  *              accepted by fdlbm_batch_add or fdlbm_step_noalloc (its step needs the handle's
  *              moment buffer). */
 
@@ -231,15 +234,18 @@ int fdlbm_save(fdlbm_t h, const char* path);
 int fdlbm_load(fdlbm_t h, const char* path);
 
 /* Launch variants of the fused step (CTA tile shapes). Every variant gives bitwise identical
- * results: a node's arithmetic does not depend on the tiling. FDLBM_FNEQ32 has its own kernel and
+ * results: a node's arithmetic does not depend on the tiling. The numbers name FP32 storage's shapes;
+ * FDLBM_FP64 serves them with five (csrc/fdlbm_step_f64.cu: 4x4 for variant 9, 8x4 for 3 and 8 and, but for 9,
+ * on every grid of up to 40960 sites, 32x4, and 32x8 at two register caps). FDLBM_FNEQ32 has its own kernel and
  * maps the variants onto its tile shapes (32x4, 32x8 at two register caps, 16x16, 64x4). Variant
  * 12 is, for FP32 storage, the 32x8 tile whose 36x12x33 box of f (tile, halo, all planes)
  * arrives in shared memory by one tensor-memory-accelerator copy; other precisions run the plain
  * 32x8 tile for it. Variants 13 and 14 (FP64 and FP32 storage) are persistent: one cooperative
  * launch runs all the steps of an fdlbm_step call (up to 4096 per launch), the CTAs meeting at a
- * grid barrier between steps, with the tile bodies of variants 9 (ring-parallel 8x4) and 2 (32x16).
- * That removes the per-step launch cost, 3% of a 1600-site step (small grids wait on the FP64 pipe
- * of their few warps, not on launches); the autotuner times them on small grids. A solve with boundary
+ * grid barrier between steps, with the tile bodies of variants 9 and 2. That saves the
+ * per-step launch and costs a barrier: 400 x 4 takes 11.0 us per step for 11.8 with FP32 storage and
+ * 10.5 for 10.7 with FP64, whose launches overlap; larger grids mostly lose (4000 x 4, FP64: 30.0 and
+ * 39.9 us against 28.6). The autotuner times them on small grids. A solve with boundary
  * segments, other precisions and fdlbm_step_noalloc run the one-step variants 9 and 2 for them. A
  * barrier wait that gives up (bounded at about 2^22 polls) sets FDLBM_HEALTH_TIMEOUT. Variant 15
  * (FP64 and FP32 storage) launches variant 9's step from CUDA graphs of 32 steps, captured the
@@ -251,7 +257,8 @@ int fdlbm_set_variant(fdlbm_t h, int variant);  /* FDLBM_E_ARG if out of range *
 int fdlbm_get_variant(fdlbm_t h);               /* current variant, or a negative status */
 
 /* Autotuner: time every variant over trial_steps steps on the current state and keep the
- * fastest. The state is not advanced. On grids of up to 262144 sites every variant is timed over at
+ * fastest (variants that run one kernel are timed once, and the first of them stands for all). The
+ * state is not advanced. On grids of up to 262144 sites every variant is timed over at
  * least 32 steps that alternate the buffers as fdlbm_step does (steps of tens of microseconds, where
  * launching and the persistent variants' start-up count), from a copy of the state and health word
  * that is restored after each variant (device memory for the copy: one state buffer). On larger

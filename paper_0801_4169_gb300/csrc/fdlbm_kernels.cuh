@@ -17,8 +17,9 @@
 // (STAGE), so that each warp's FP64 work comes in one dense stretch.
 //
 // On this GPU an FP64 instruction (including an FP32<->FP64 conversion) issues at 2/clk/SM, ~64x
-// below FP32, so the step is bound by the FP64 pipe, not by HBM. The code is arranged to issue as
-// few FP64 operations per node as the method allows:
+// below FP32: with its sums in FP64 the step was bound by that pipe (86% busy), now by instruction issue (55%,
+// half of it integer multiply-adds), and never by HBM. The code is arranged to issue as few FP64 operations
+// per node as the method allows:
 //   * ring moments from shared differences (S, X, Y per ring: 15 ops with FP64 storage); with
 //     FP32 storage the ring, speed-weighted momentum and energy sums are exact 64-bit integers,
 //     and only sqrt(1/2), the two energy parts' sum and 1/100, 10^-4 are applied in FP64;

@@ -60,7 +60,8 @@ cudaError_t launch_batch_fx(const BatchMember* mem, int nmem, long long n, unsig
 // Five shapes serve the variants: every shape gives the same bits, and a larger tile than 32 x 8 does not
 // fit its planes and powers twice per SM. On a grid of up to kF64SmallSites the large tiles leave most SMs idle
 // (400 x 4: 40 us per step against 13.9 with 8 x 4 tiles; 200 x 200: 62.6 against 52.6), so it gets the 8 x 4
-// tile instead; at 333 x 333 it is 121 against 94.
+// tile instead; at 333 x 333 it is 121 against 94. The 32 x 8 shape at three CTAs per SM spills (2048 x 2048: 2.48 against
+// 2.43 ms per step), but takes 305 to 456 tiles in one wave instead of two (500 x 200: 83 against 87 us).
 cudaError_t launch_step_f64(int variant, const void* f, void* fn, const Grid& g, const Coeffs& c, unsigned* health,
                           cudaStream_t s) {
   switch (variant_kernel(FDLBM_FP64, variant, (long long)g.nx * g.ny)) {
