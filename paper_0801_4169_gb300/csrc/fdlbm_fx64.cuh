@@ -322,9 +322,10 @@ __device__ __forceinline__ bool finish(const Acc& a, s64 B, int ex, int unit, do
 }
 
 // A plane of several classes: a stencil's first NP cells, FP64 numbers, become integers of their largest class cl,
-// m 2^(6 - s) with s = 4 cl + 1 - E, rounded to nearest even: a rounding of one sign would add up. FP64 numbers in the
+// m 2^(6 - s) with s = 4 cl + 1 - E, rounded to odd as in mom_term: a rounding of one sign would add up. FP64 numbers in the
 // box and not integers of 15 classes below the plane's largest, since no span of a tile's values may change a stencil's:
-// 1023 x 777 497 us per step against 503, a 32-tube batch 23.0 ms against 23.6, 400 x 4 10.4 us against 10.0.
+// 1023 x 777 497 us per step against 503, a 32-tube batch 23.0 ms against 23.6, 400 x 4 10.4 us against 10.0. To nearest
+// even instead the double Mach reflection's pass takes 2242 us, not 2175, and a 9000 x 4 tube's 3209, not 3148.
 template <int NP>
 __device__ __forceinline__ void align_cells(int2 (&t)[9], int& cl) {
   unsigned top = 0u;
@@ -334,9 +335,10 @@ __device__ __forceinline__ void align_cells(int2 (&t)[9], int& cl) {
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const unsigned hi = (unsigned)t[i].y, lo = (unsigned)t[i].x, m = (hi & 0xfffffu) | 0x100000u;
-    const int s = min(4 * cl + 1 - (int)((hi & 0x7fffffffu) >> 20), 63);  // 1..; of a zero 63, which leaves nothing
-    const u64 v = ((u64)__funnelshift_l(lo, m, 6) << 32) | (lo << 6);
-    const u64 r = (v + ((1ull << (s - 1)) - 1ull) + ((v >> s) & 1ull)) >> s;
+    const int s = 4 * cl + 1 - (int)((hi & 0x7fffffffu) >> 20);  // 1..; of a zero so large that nothing is left
+    const unsigned l6 = lo << 6;
+    const u64 r = fx::shr_clamped(((u64)__funnelshift_l(lo, m, 6) << 32) | l6, s) |
+                  (fx::shl_clamped(l6, max(32 - s, 0)) ? 1u : 0u);
     const s64 sg = (s64)((int)hi >> 31);
     const L28 u = l28((s64)(r ^ (u64)sg) - sg);
     t[i] = make_int2(u.h, u.l);
