@@ -262,10 +262,11 @@ int default_variant(const fdlbm_config* c) {
   if (c->prec == FDLBM_FNEQ32) return c->ny <= 4 ? V_T32x4 : V_T32x8;  // its own kernel (fdlbm_fneq.cu)
   if (c->prec == FDLBM_FP32_STORE_DW) return V_TMA32x8;  // fastest at every size measured (tiny grids: 32 x 8)
   if (c->prec == FDLBM_FP64) {
-    // Times per step on a GB300 (us). The 4 x 4 tile (V_RP8x4; two per SM, 4864 sites at a time) is the shortest
-    // step: 400 x 4 9.7 against 13.9 with 8 x 4 tiles, 2000 x 4 18.4 against 22.6; in its third round, at 4000 x 4,
-    // 32.9 against 23.6. The 8 x 4 tile holds 19456 sites at a time: 200 x 200 52.6 against 62.6 with 32 x 8 tiles,
-    // 16384 x 4 74.2 against 53.0 with 32 x 4. Beyond, 32 x 8 (2048^2 2170, 32 x 4 2540), a tube's 4 rows 32 x 4.
+    // Times per step on a GB300 (us, a smooth periodic state). The 4 x 4 tile (V_RP8x4; two per SM, 4864 sites at a
+    // time) is the shortest step: 400 x 4 10.7 against 14.7 with 8 x 4 tiles, 2000 x 4 20.6 against 27.1; in its third
+    // round, at 4000 x 4, 36.4 against 28.6. The 8 x 4 tile holds 19456 sites at a time: 200 x 200 57.8 (a four-quadrant
+    // state 52.6 against 62.6 with 32 x 8 tiles), 16384 x 4 89.3 against 61.0 with 32 x 4. Beyond, 32 x 8 (1023 x 777
+    // 502, 32 x 4 661), a tube's 4 rows 32 x 4.
     if (sites <= 9728) return V_RP8x4;
     if (sites <= kF64SmallSites) return V_RP16x4;
     return c->ny <= 4 ? V_T32x4 : V_T32x16;
